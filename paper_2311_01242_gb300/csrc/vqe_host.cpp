@@ -104,6 +104,18 @@ void parallel_items(int64_t n, F f) {
   for (auto& t : ts) t.join();
 }
 
+// Run f(lo, hi) over [0, n) in short ranges on all threads (items of large cost,
+// such as the strings of a sector).
+template <typename F>
+void parallel_ranges(int64_t n, F f) {
+  constexpr int64_t step = 16;
+  if (n < 8 * step) {
+    f(int64_t(0), n);
+    return;
+  }
+  parallel_items((n + step - 1) / step, [&](int64_t i) { f(i * step, std::min(n, (i + 1) * step)); });
+}
+
 // ------------------------------------------------------------------ Pauli algebra
 // A Pauli string P(x, z) = i^{|x&z|} X^x Z^z. Product rule:
 // P(x1,z1) P(x2,z2) = i^{|x1&z1| + |x2&z2| + 2|z1&x2| - |x&z|} P(x, z), x = x1^x2, z = z1^z2.
@@ -290,7 +302,11 @@ struct vqe_hamiltonian_s {
     bool use_str = false;
     vqe::StrPlan str{};
     vqe::StrPlan* d_str = nullptr;     // device copy of str (batched kernels)
-    std::vector<void*> str_alloc;      // device arrays behind str
+    std::vector<void*> str_alloc;      // device arrays behind str, rest and tc
+    // large sectors: hop x hop groups on the tensor cores, the others in `rest`
+    bool use_tc = false, has_rest = false;
+    vqe::TcPlan tc{};
+    vqe::StrPlan rest{};
   };
   std::mutex mu;
   std::map<std::tuple<int, int, int>, Ell> ells;
@@ -522,70 +538,39 @@ double fp64_adds(vqe_hamiltonian_t h, int g, uint32_t src) {
   return r.kind == 1 ? double(k) : double(k + k * (k - 1) / 2);
 }
 
-// String tables of a spin sector (the product of alpha strings on the even
-// qubits and beta strings on the odd qubits) for the string-driven H psi:
-//  - alpha and beta strings in increasing order, and the alpha-major order's
-//    map to the sector's sorted order (perm);
-//  - groups that can connect anything (even numbers of flipped alpha and beta
-//    bits) in buckets of equal alpha mask, each bucket sorted by beta mask;
-//  - for each output alpha string and bucket, the source alpha string (or -1);
-//  - for each beta mask, the (output, source) beta string pairs in output
-//    order, with the entry range of each warp's fixed share of outputs.
-int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e) {
-  const int n = a->n, Na = a->n_alpha, Nb = a->n_elec - a->n_alpha;
-  const uint32_t all = uint32_t((uint64_t(1) << n) - 1);
-  const uint32_t even = all & 0x55555555u, odd = all & 0xAAAAAAAAu;
-  auto subsets = [](uint32_t pool, int c) {
-    std::vector<uint32_t> bits, out;
-    for (int q = 0; q < 32; ++q)
-      if ((pool >> q) & 1u) bits.push_back(q);
-    const int m = int(bits.size());
-    if (c < 0 || c > m) return out;
-    // every c-subset of the pool, as masks, in increasing order
-    std::vector<uint32_t> all_masks;
-    for (uint64_t v = 0; v < (uint64_t(1) << m); ++v) {
-      if (__builtin_popcountll(v) != c) continue;
-      uint32_t w = 0;
-      for (int j = 0; j < m; ++j)
-        if ((v >> j) & 1) w |= 1u << bits[j];
-      all_masks.push_back(w);
-    }
-    std::sort(all_masks.begin(), all_masks.end());
-    return all_masks;
-  };
-  const std::vector<uint32_t> ka = subsets(even, Na), kb = subsets(odd, Nb);
+// The strings of a spin sector, shared by every table built over them.
+struct Strings {
+  std::vector<uint32_t> ka, kb;
+  uint32_t even = 0, odd = 0;
+  int Na = 0, Nb = 0;
+  uint32_t *d_ka = nullptr, *d_kb = nullptr, *d_perm = nullptr;
+};
+int32_t index_of(const std::vector<uint32_t>& v, uint32_t m) {
+  auto it = std::lower_bound(v.begin(), v.end(), m);
+  return (it != v.end() && *it == m) ? int32_t(it - v.begin()) : -1;
+}
+// bits of `pool` strictly between the two bits of a hop mask (0 when it is no hop)
+uint32_t between(uint32_t x2, uint32_t pool) {
+  if (pc32(x2) != 2) return 0u;
+  const int lo_q = __builtin_ctz(x2), hi_q = 31 - __builtin_clz(x2);
+  return ((1u << hi_q) - 1u) & ~((2u << lo_q) - 1u) & pool;
+}
+template <typename T>
+int upload_str(vqe_hamiltonian_s::Ell* e, const std::vector<T>& vec, T** dst) {
+  const int r = upload(vec, dst);
+  if (r == VQE_OK) e->str_alloc.push_back(static_cast<void*>(*dst));
+  return r;
+}
+
+// String-driven tables of the groups in `keep` (see StrPlan). *built is false
+// when they would be too large.
+int build_buckets(vqe_hamiltonian_t h, const Strings& S, std::vector<int> keep, vqe_hamiltonian_s::Ell* e,
+                  vqe::StrPlan* plan, bool* built) {
+  const std::vector<uint32_t>&ka = S.ka, &kb = S.kb;
   const int64_t Da = int64_t(ka.size()), Db = int64_t(kb.size());
-  // shared memory of a block (complex amplitudes: the larger of the two)
-  const size_t smem = vqe::str_smem_bytes(int(std::min<int64_t>(Db, 65535)), 16);
-  if (Da * Db != int64_t(a->sector.size()) || Db > 8191 || smem > size_t(200) * 1024) return VQE_OK;  // not used
-  {
-    static std::mutex mu;
-    static size_t set_to = 0;
-    std::lock_guard<std::mutex> lk(mu);
-    if (smem > set_to) {
-      const cudaError_t ce = vqe::set_str_smem_limit(smem);
-      if (ce != cudaSuccess) return cuda_fail(ce, "string-driven H psi shared memory");
-      set_to = smem;
-    }
-  }
-  auto index_of = [](const std::vector<uint32_t>& v, uint32_t m) -> int32_t {
-    auto it = std::lower_bound(v.begin(), v.end(), m);
-    return (it != v.end() && *it == m) ? int32_t(it - v.begin()) : -1;
-  };
-  const uint32_t lo_mask = (1u << a->lo_bits) - 1u;
-  auto rank = [&](uint32_t k) { return a->rank_hi[k >> a->lo_bits] + a->rank_lo[k & lo_mask]; };
-  std::vector<uint32_t> perm(size_t(Da * Db));
-  parallel_for(Da, [&](int64_t lo, int64_t hi) {
-    for (int64_t i = lo; i < hi; ++i)
-      for (int64_t j = 0; j < Db; ++j) perm[size_t(i * Db + j)] = rank(ka[size_t(i)] | kb[size_t(j)]);
-  });
-  // buckets of groups by alpha mask, each sorted by beta mask then index
-  const int G = int(h->groups.size());
-  std::vector<int> keep;
-  for (int g = 0; g < G; ++g) {
-    const uint32_t x = h->groups[g].x;
-    if ((pc32(x & even) & 1) == 0 && (pc32(x & odd) & 1) == 0) keep.push_back(g);
-  }
+  const uint32_t even = S.even, odd = S.odd;
+  const int Na = S.Na, Nb = S.Nb;
+  *built = false;
   std::stable_sort(keep.begin(), keep.end(), [&](int p, int q) {
     const uint32_t xp = h->groups[p].x, xq = h->groups[q].x;
     if ((xp & even) != (xq & even)) return (xp & even) < (xq & even);
@@ -611,7 +596,7 @@ int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e
   const int NB = int(bxa.size()), NL = int(lxb.size());
   // source alpha string per (output alpha string, bucket)
   std::vector<int32_t> ja(size_t(Da) * size_t(std::max(NB, 1)), -1);
-  parallel_for(Da, [&](int64_t lo, int64_t hi) {
+  parallel_ranges(Da, [&](int64_t lo, int64_t hi) {
     for (int64_t i = lo; i < hi; ++i)
       for (int b = 0; b < NB; ++b) {
         const uint32_t src = ka[size_t(i)] ^ bxa[size_t(b)];
@@ -625,17 +610,17 @@ int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e
   // single hop {q_lo < q_hi}, bit 13 says the source string holds q_hi (else q_lo)
   // and bit 14 is the parity of the source's beta qubits strictly between them
   std::vector<std::vector<uint32_t>> lists(static_cast<size_t>(NL));
-  parallel_for(NL, [&](int64_t lo, int64_t hi) {
+  parallel_ranges(NL, [&](int64_t lo, int64_t hi) {
     for (int64_t l = lo; l < hi; ++l) {
       const uint32_t xb = lxb[size_t(l)];
       const bool hop = pc32(xb) == 2;
       const int q_lo = hop ? __builtin_ctz(xb) : 0, q_hi = hop ? 31 - __builtin_clz(xb) : 0;
-      const uint32_t between = hop ? (((1u << q_hi) - 1u) & ~((2u << q_lo) - 1u) & odd) : 0u;
+      const uint32_t inside = hop ? between(xb, odd) : 0u;
       for (int64_t j = 0; j < Db; ++j) {
         const uint32_t src = kb[size_t(j)] ^ xb;
         if (pc32(src) != Nb) continue;
         uint32_t ent = uint32_t(j) | (uint32_t(index_of(kb, src)) << 16);
-        if (hop) ent |= ((src >> q_hi) & 1u) << 13 | uint32_t(pc32(src & between) & 1) << 14;
+        if (hop) ent |= ((src >> q_hi) & 1u) << 13 | uint32_t(pc32(src & inside) & 1) << 14;
         lists[size_t(l)].push_back(ent);
       }
     }
@@ -666,11 +651,7 @@ int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e
   }
   // per bucket: for a single alpha hop {p < q}, the beta qubits strictly between
   // p and q; the bucket's staged source row is multiplied by (-1)^{|Jb & bob|}
-  auto between_odd = [&](uint32_t x2) -> uint32_t {
-    if (pc32(x2) != 2) return 0u;
-    const int lo_q = __builtin_ctz(x2), hi_q = 31 - __builtin_clz(x2);
-    return ((1u << hi_q) - 1u) & ~((2u << lo_q) - 1u) & odd;
-  };
+  auto between_odd = [&](uint32_t x2) { return between(x2, odd); };
   std::vector<uint32_t> bob(size_t(std::max(NB, 1)), 0u);
   for (int b = 0; b < NB; ++b) bob[size_t(b)] = between_odd(bxa[size_t(b)]);
   std::vector<int32_t> bucket_of(bgrp.size(), 0);
@@ -709,38 +690,410 @@ int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e
     bgx[i] = make_uint4(qa, qb, uint32_t(g.vbeg) | (single ? 0x80000000u : 0u), single ? h->emask[size_t(g.ebeg)] : 0u);
   }
   if (bgx.empty()) bgx.push_back(make_uint4(0xFFFFFFFFu, 0u, 0u, 0u));
-  vqe::StrPlan& P = e->str;
+  vqe::StrPlan& P = *plan;
   P.Da = int32_t(Da);
   P.Db = int32_t(Db);
   P.NB = NB;
   int rc;
-  auto up = [&](auto& vec, auto** dst) -> int {
-    int r = upload(vec, dst);
-    if (r == VQE_OK) e->str_alloc.push_back(static_cast<void*>(*dst));
-    return r;
-  };
-  uint32_t *d_ka, *d_kb, *d_lists, *d_perm;
+  uint32_t* d_lists;
   int32_t *d_ja, *d_boff, *d_bgrp, *d_bsplit;
   uint4* d_bgx;
   uint32_t* d_bob;
-  std::vector<uint32_t> ka_v(ka), kb_v(kb);
-  if ((rc = up(ka_v, &d_ka)) || (rc = up(kb_v, &d_kb)) || (rc = up(ja, &d_ja)) || (rc = up(boff, &d_boff)) ||
-      (rc = up(bgrp, &d_bgrp)) || (rc = up(bsplit, &d_bsplit)) || (rc = up(flat, &d_lists)) ||
-      (rc = up(perm, &d_perm)) || (rc = up(bgx, &d_bgx)) || (rc = up(bob, &d_bob)))
+  if ((rc = upload_str(e, ja, &d_ja)) || (rc = upload_str(e, boff, &d_boff)) || (rc = upload_str(e, bgrp, &d_bgrp)) ||
+      (rc = upload_str(e, bsplit, &d_bsplit)) || (rc = upload_str(e, flat, &d_lists)) ||
+      (rc = upload_str(e, bgx, &d_bgx)) || (rc = upload_str(e, bob, &d_bob)))
     return rc;
   P.bgx = d_bgx;
   P.bob = d_bob;
-  P.ka = d_ka;
-  P.kb = d_kb;
+  P.ka = S.d_ka;
+  P.kb = S.d_kb;
   P.ja = d_ja;
   P.boff = d_boff;
   P.bgrp = d_bgrp;
   P.bsplit = d_bsplit;
   P.lists = d_lists;
-  P.perm = d_perm;
-  std::vector<vqe::StrPlan> one(1, P);
+  P.perm = S.d_perm;
+  *built = true;
+  return VQE_OK;
+}
+
+// Sectors from this size on evaluate their hop x hop groups on the tensor cores.
+// (Smaller ones also run inside the batch's persistent launch, whose results equal
+// the single calls' bit for bit.)
+constexpr int64_t kTcMinStates = int64_t(vqe::kMaxPartials) * vqe::kStreamThreads + 1;
+
+// How the tensor-core H psi takes a group. Amplitudes are multiplied by s(Ia, Ib) =
+// (-1)^{alpha electrons above beta ones}; a group is taken when its sign then
+// splits into the hops' own signs (the parity of the electrons of that spin between
+// the hop's qubits), or for two-electron moves into a sign of that spin's string,
+// up to a constant that the source's occupation of the hop qubits fixes. This holds
+// for every group of a Jordan-Wigner Hamiltonian; others stay string-driven.
+enum class TcKind { kNone, kHopHop, kHopA, kHopB, kMoveA, kMoveB, kDiag };
+TcKind tc_kind(vqe_hamiltonian_t h, const Strings& S, const GroupRec& g) {
+  const uint32_t xa = g.x & S.even, xb = g.x & S.odd, em = h->emask[size_t(g.ebeg)];
+  const int na = pc32(xa), nb = pc32(xb);
+  const bool single = g.kind == 0 && g.eend == g.ebeg + 1;
+  if (na == 0 && nb == 0) return g.kind == 2 && em == 0 ? TcKind::kDiag : TcKind::kNone;
+  // qubits of the other spin below (above) an odd number of flipped ones
+  uint32_t below = 0, above = 0;
+  for (uint32_t m = xa; m; m &= m - 1) below ^= ((m & (0u - m)) - 1u) & S.odd;
+  for (uint32_t m = xb; m; m &= m - 1) above ^= ~(((m & (0u - m)) << 1) - 1u) & S.even;
+  if (na == 2 && nb == 2) {
+    const uint32_t ra = (em & S.even) ^ above ^ between(xa, S.even);
+    const uint32_t rb = (em & S.odd) ^ below ^ between(xb, S.odd);
+    return single && g.ubits == 4 && (ra & ~xa) == 0 && (rb & ~xb) == 0 ? TcKind::kHopHop : TcKind::kNone;
+  }
+  if (na == 2 && nb == 0)
+    return g.kind == 1 && g.ubits == 2 && em == (below | between(xa, S.even)) ? TcKind::kHopA : TcKind::kNone;
+  if (na == 0 && nb == 2)
+    return g.kind == 1 && g.ubits == 2 && em == (above | between(xb, S.odd)) ? TcKind::kHopB : TcKind::kNone;
+  if (na == 4 && nb == 0) return single && g.ubits == 4 && (em & S.odd) == below ? TcKind::kMoveA : TcKind::kNone;
+  if (na == 0 && nb == 4) return single && g.ubits == 4 && (em & S.even) == above ? TcKind::kMoveB : TcKind::kNone;
+  return TcKind::kNone;
+}
+
+uint32_t pattern_bits(const GroupRec& g, uint32_t src) {
+  uint32_t u = 0;
+  for (int j = 0; j < g.ubits; ++j) u |= ((src >> ((g.upos >> (8 * j)) & 31u)) & 1u) << j;
+  return u;
+}
+
+// One spin's matrix (TcOneSpin): the moves, single hops and diagonal terms that
+// touch that spin only, for strings `k` of `count` electrons on the qubits `pool`.
+int build_one_spin(vqe_hamiltonian_t h, const std::vector<uint32_t>& k, uint32_t pool, int count,
+                   const std::vector<int>& hops, const std::vector<int>& moves, int diag, bool with_const,
+                   vqe_hamiltonian_s::Ell* e, vqe::TcOneSpin* out) {
+  const int64_t n = int64_t(k.size());
+  struct Row {
+    std::vector<int32_t> col, len;
+    std::vector<uint32_t> slot;
+  };
+  std::vector<Row> rows(static_cast<size_t>(n));
+  parallel_ranges(n, [&](int64_t lo, int64_t hi) {
+    for (int64_t i = lo; i < hi; ++i) {
+      Row& r = rows[size_t(i)];
+      const uint32_t ki = k[size_t(i)];
+      auto end = [&](int32_t col, size_t before) {
+        r.col.push_back(col);
+        r.len.push_back(int32_t(r.slot.size() - before));
+      };
+      if (diag >= 0) {
+        const GroupRec& g = h->groups[size_t(diag)];
+        const size_t before = r.slot.size();
+        const uint32_t q0 = uint32_t(g.vbeg), nq = uint32_t(g.nq);
+        if (with_const) r.slot.push_back(q0);
+        const uint32_t m = ki & h->emask[size_t(g.ebeg) + 1];
+        for (uint32_t a = m; a; a &= a - 1) {
+          const uint32_t p = uint32_t(__builtin_ctz(a));
+          r.slot.push_back(q0 + 1 + p);
+          for (uint32_t c = a & (a - 1); c; c &= c - 1)
+            r.slot.push_back(q0 + 1 + nq + p * nq + uint32_t(__builtin_ctz(c)));
+        }
+        end(int32_t(i), before);
+      }
+      for (int gi : hops) {
+        const GroupRec& g = h->groups[size_t(gi)];
+        const uint32_t src = ki ^ (g.x & pool);
+        if (pc32(src) != count) continue;
+        const size_t before = r.slot.size();
+        const uint32_t s = uint32_t(pc32(src & h->emask[size_t(g.ebeg)]) & 1) << 31, u = pattern_bits(g, src);
+        r.slot.push_back((uint32_t(g.vbeg) + u) | s);
+        for (uint32_t a = src & h->emask[size_t(g.ebeg) + 1]; a; a &= a - 1)
+          r.slot.push_back((uint32_t(g.vbeg) + (uint32_t(1 + __builtin_ctz(a)) << g.ubits) + u) | s);
+        end(index_of(k, src), before);
+      }
+      for (int gi : moves) {
+        const GroupRec& g = h->groups[size_t(gi)];
+        const uint32_t src = ki ^ (g.x & pool);
+        if (pc32(src) != count) continue;
+        const size_t before = r.slot.size();
+        r.slot.push_back((uint32_t(g.vbeg) + pattern_bits(g, src)) |
+                         (uint32_t(pc32(src & h->emask[size_t(g.ebeg)]) & 1) << 31));
+        end(index_of(k, src), before);
+      }
+    }
+  });
+  std::vector<int32_t> off(1, 0), col, soff(1, 0);
+  std::vector<uint32_t> slot;
+  for (const Row& r : rows) {
+    col.insert(col.end(), r.col.begin(), r.col.end());
+    for (int32_t l : r.len) soff.push_back(soff.back() + l);
+    slot.insert(slot.end(), r.slot.begin(), r.slot.end());
+    if (slot.size() > size_t(INT32_MAX / 2)) return fail(VQE_ERR_INVALID_ARG, "one-spin table too large");
+    off.push_back(int32_t(col.size()));
+  }
+  if (col.empty()) {
+    col.push_back(0);
+    slot.push_back(0);
+  }
+  int rc;
+  int32_t *d_off, *d_col, *d_soff;
+  uint32_t* d_slot;
+  if ((rc = upload_str(e, off, &d_off)) || (rc = upload_str(e, col, &d_col)) || (rc = upload_str(e, soff, &d_soff)) ||
+      (rc = upload_str(e, slot, &d_slot)))
+    return rc;
+  out->n = int32_t(n);
+  out->off = d_off;
+  out->col = d_col;
+  out->soff = d_soff;
+  out->slot = d_slot;
+  return VQE_OK;
+}
+
+// Tables of the tensor-core H psi (TcPlan) and, for the groups it does not take, of
+// the string-driven one (Ell::rest).
+int build_tc(vqe_hamiltonian_t h, const Strings& S, const std::vector<int>& keep, vqe_hamiltonian_s::Ell* e) {
+  const int64_t Da = int64_t(S.ka.size()), Db = int64_t(S.kb.size());
+  const int n = h->n;
+  if (Da * Db < kTcMinStates) return VQE_OK;
+  int dev = 0, optin = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return VQE_OK;
+  // rows: beta hops, then beta qubits; items: directed alpha hops, then alpha qubits
+  std::vector<uint32_t> ha, hb;
+  std::map<uint32_t, int> na, nb;
+  for (int q = 0; q < n; ++q)
+    for (int r = q + 2; r < n; r += 2) {
+      const uint32_t x = (1u << q) | (1u << r);
+      auto& v = (q & 1) ? hb : ha;
+      ((q & 1) ? nb : na)[x] = int(v.size());
+      v.push_back(x);
+    }
+  const int qa = (n + 1) / 2, qb = n / 2;
+  auto item_of = [&](uint32_t x, int up) { return 2 * na[x] + up; };
+  auto diag_item = [&](int q) { return 2 * int(ha.size()) + q / 2; };
+  auto diag_row = [&](int q) { return int(hb.size()) + q / 2; };
+  vqe::TcPlan T;
+  std::memset(&T, 0, sizeof(T));
+  T.MT = (int(hb.size()) + qb + 127) / 128;
+  const int R = T.MT * 128, zero_item = 2 * int(ha.size()) + qa;
+  T.items = zero_item + 1;
+  if (T.MT < 1 || T.items > 65535) return VQE_OK;
+  std::vector<int2> vslot(size_t(T.items) * R, make_int2(-1, -1));
+  std::vector<char> used(size_t(T.items), 0);
+  auto set = [&](int item, int row, uint32_t lower, uint32_t upper) {
+    used[size_t(item)] = 1;
+    vslot[size_t(item) * R + row] = make_int2(int(lower), int(upper));
+  };
+  auto ends = [](uint32_t x, int up) { return up ? 31 - __builtin_clz(x) : __builtin_ctz(x); };
+  std::vector<int> rest, hops_a, hops_b, moves_a, moves_b;
+  int diag = -1;
+  for (int gi : keep) {
+    const GroupRec& g = h->groups[size_t(gi)];
+    const uint32_t xa = g.x & S.even, xb = g.x & S.odd;
+    const uint32_t em = h->emask[size_t(g.ebeg)], v0 = uint32_t(g.vbeg);
+    switch (tc_kind(h, S, g)) {
+      case TcKind::kHopHop: {
+        const uint32_t ra = (em & S.even) ^ between(xb, S.even) ^ between(xa, S.even);
+        const uint32_t rb = (em & S.odd) ^ between(xa, S.odd) ^ between(xb, S.odd);
+        const int flip = pc32(xb & between(xa, S.odd)) & 1;
+        for (int da = 0; da < 2; ++da) {
+          uint32_t slot[2];
+          for (int db = 0; db < 2; ++db) {
+            const uint32_t src = (1u << ends(xa, da)) | (1u << ends(xb, db));
+            slot[db] = (v0 + pattern_bits(g, src)) | uint32_t(flip ^ (pc32(src & (ra | rb)) & 1)) << 31;
+          }
+          set(item_of(xa, da), nb[xb], slot[0], slot[1]);
+        }
+        break;
+      }
+      case TcKind::kHopA:
+        hops_a.push_back(gi);
+        for (int da = 0; da < 2; ++da)
+          for (uint32_t m = h->emask[size_t(g.ebeg) + 1] & S.odd; m; m &= m - 1) {
+            const int q = __builtin_ctz(m);
+            const uint32_t sl = v0 + (uint32_t(1 + q) << g.ubits) + pattern_bits(g, 1u << ends(xa, da));
+            set(item_of(xa, da), diag_row(q), sl, sl);
+          }
+        break;
+      case TcKind::kHopB:
+        hops_b.push_back(gi);
+        for (uint32_t m = h->emask[size_t(g.ebeg) + 1] & S.even; m; m &= m - 1) {
+          const int q = __builtin_ctz(m);
+          const uint32_t sl = v0 + (uint32_t(1 + q) << g.ubits);
+          set(diag_item(q), nb[xb], sl + pattern_bits(g, 1u << ends(xb, 0)), sl + pattern_bits(g, 1u << ends(xb, 1)));
+        }
+        break;
+      case TcKind::kMoveA: moves_a.push_back(gi); break;
+      case TcKind::kMoveB: moves_b.push_back(gi); break;
+      case TcKind::kDiag: {
+        diag = gi;  // one group has x = 0
+        const uint32_t occ = h->emask[size_t(g.ebeg) + 1], q0 = v0 + 1 + uint32_t(g.nq);
+        for (uint32_t m = occ & S.even; m; m &= m - 1)
+          for (uint32_t w = occ & S.odd; w; w &= w - 1) {
+            const int p = __builtin_ctz(m), q = __builtin_ctz(w);
+            const uint32_t sl = q0 + uint32_t(std::min(p, q)) * uint32_t(g.nq) + uint32_t(std::max(p, q));
+            set(diag_item(p), diag_row(q), sl, sl);
+          }
+        break;
+      }
+      case TcKind::kNone: rest.push_back(gi); break;
+    }
+  }
+  if (rest.size() == keep.size()) return VQE_OK;
+  // sources of every output alpha string
+  std::vector<std::vector<std::pair<uint32_t, uint16_t>>> src(static_cast<size_t>(Da));
+  parallel_ranges(Da, [&](int64_t lo, int64_t hi) {
+    for (int64_t i = lo; i < hi; ++i) {
+      auto& v = src[size_t(i)];
+      const uint32_t ki = S.ka[size_t(i)];
+      for (size_t x = 0; x < ha.size(); ++x) {
+        const uint32_t j = ki ^ ha[x];
+        if (pc32(j) != S.Na) continue;
+        const int item = 2 * int(x) + int((j >> (31 - __builtin_clz(ha[x]))) & 1u);
+        if (!used[size_t(item)]) continue;
+        const uint32_t s = uint32_t(pc32(j & between(ha[x], S.even)) & 1);
+        v.push_back({uint32_t(index_of(S.ka, j)) | (s << 31), uint16_t(item)});
+      }
+      for (uint32_t m = ki; m; m &= m - 1) {
+        const int item = diag_item(__builtin_ctz(m));
+        if (used[size_t(item)]) v.push_back({uint32_t(i), uint16_t(item)});
+      }
+    }
+  });
+  for (const auto& v : src) T.K = std::max(T.K, int32_t(v.size()));
+  if (T.K == 0) return VQE_OK;
+  T.Da = int32_t(Da);
+  T.Db = int32_t(Db);
+  T.DaP = int32_t((Da + 63) / 64 * 64);
+  T.DbP = int32_t((Db + 63) / 64 * 64);
+  T.chunks = (T.K + 63) / 64;
+  T.KT = 64 * T.chunks;
+  T.sms = sms;
+  T.stages = vqe::tc_stages(T.DbP, size_t(optin));
+  if (T.stages == 0 || size_t(std::max(T.DaP, T.DbP)) * 8 + 2048 > size_t(optin)) return VQE_OK;
+  std::vector<uint32_t> kj(size_t(Da) * T.KT);
+  std::vector<uint16_t> kit(size_t(Da) * T.KT, uint16_t(zero_item));
+  for (int64_t i = 0; i < Da; ++i)
+    for (int k = 0; k < T.KT; ++k) {
+      const auto& v = src[size_t(i)];
+      kj[size_t(i * T.KT + k)] = k < int(v.size()) ? v[size_t(k)].first : uint32_t(i);
+      if (k < int(v.size())) kit[size_t(i * T.KT + k)] = v[size_t(k)].second;
+    }
+  std::vector<uint4> dst(size_t(T.DbP) / 8 * R, make_uint4(0, 0, 0, 0));
+  auto put = [&](int64_t j, int row, uint32_t v) {  // halfword j % 8
+    uint32_t* w = &dst[size_t(j / 8) * R + size_t(row)].x;
+    w[(j & 7) >> 1] |= v << (16 * (j & 1));
+  };
+  parallel_ranges(T.DbP / 8, [&](int64_t lo, int64_t hi) {  // eight strings share a word
+    for (int64_t j = lo * 8; j < std::min(hi * 8, Db); ++j) {
+      const uint32_t kj_ = S.kb[size_t(j)];
+      for (size_t x = 0; x < hb.size(); ++x) {
+        const uint32_t i = kj_ ^ hb[x];
+        if (pc32(i) != S.Nb) continue;
+        const uint32_t up = (kj_ >> (31 - __builtin_clz(hb[x]))) & 1u;
+        const uint32_t s = uint32_t(pc32(kj_ & between(hb[x], S.odd)) & 1);
+        put(j, int(x), uint32_t(index_of(S.kb, i)) | (s << 13) | (up << 14) | 0x8000u);
+      }
+      for (uint32_t m = kj_; m; m &= m - 1)
+        put(j, diag_row(__builtin_ctz(m)), uint32_t(j) | 0x8000u);
+    }
+  });
+  int rc;
+  if (!rest.empty()) {
+    bool ok = false;
+    if ((rc = build_buckets(h, S, rest, e, &e->rest, &ok)) != VQE_OK || !ok) return rc;
+    e->has_rest = true;
+  }
+  if ((rc = build_one_spin(h, S.ka, S.even, S.Na, hops_a, moves_a, diag, true, e, &T.alpha)) ||
+      (rc = build_one_spin(h, S.kb, S.odd, S.Nb, hops_b, moves_b, diag, false, e, &T.beta)))
+    return rc;
+  uint32_t* d_kj;
+  uint16_t* d_kit;
+  uint4* d_dst;
+  int2* d_vslot;
+  if ((rc = upload_str(e, kj, &d_kj)) || (rc = upload_str(e, kit, &d_kit)) || (rc = upload_str(e, dst, &d_dst)) ||
+      (rc = upload_str(e, vslot, &d_vslot)))
+    return rc;
+  T.kj = d_kj;
+  T.kit = d_kit;
+  T.dst = d_dst;
+  T.vslot = d_vslot;
+  const cudaError_t ce = vqe::tc_set_smem_limit(size_t(optin));
+  if (ce != cudaSuccess) return cuda_fail(ce, "tensor-core H psi shared memory");
+  e->tc = T;
+  e->use_tc = true;
+  return VQE_OK;
+}
+
+// String tables of a spin sector (the product of alpha strings on the even
+// qubits and beta strings on the odd qubits) for the string-driven H psi:
+//  - alpha and beta strings in increasing order, and the alpha-major order's
+//    map to the sector's sorted order (perm);
+//  - groups that can connect anything (even numbers of flipped alpha and beta
+//    bits) in buckets of equal alpha mask, each bucket sorted by beta mask;
+//  - for each output alpha string and bucket, the source alpha string (or -1);
+//  - for each beta mask, the (output, source) beta string pairs in output
+//    order, with the entry range of each warp's fixed share of outputs.
+int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e) {
+  const int n = a->n, Na = a->n_alpha, Nb = a->n_elec - a->n_alpha;
+  const uint32_t all = uint32_t((uint64_t(1) << n) - 1);
+  const uint32_t even = all & 0x55555555u, odd = all & 0xAAAAAAAAu;
+  auto subsets = [](uint32_t pool, int c) {
+    std::vector<uint32_t> bits, out;
+    for (int q = 0; q < 32; ++q)
+      if ((pool >> q) & 1u) bits.push_back(q);
+    const int m = int(bits.size());
+    if (c < 0 || c > m) return out;
+    // every c-subset of the pool, as masks, in increasing order
+    std::vector<uint32_t> all_masks;
+    for (uint64_t v = 0; v < (uint64_t(1) << m); ++v) {
+      if (__builtin_popcountll(v) != c) continue;
+      uint32_t w = 0;
+      for (int j = 0; j < m; ++j)
+        if ((v >> j) & 1) w |= 1u << bits[j];
+      all_masks.push_back(w);
+    }
+    std::sort(all_masks.begin(), all_masks.end());
+    return all_masks;
+  };
+  Strings S;
+  S.ka = subsets(even, Na);
+  S.kb = subsets(odd, Nb);
+  S.even = even;
+  S.odd = odd;
+  S.Na = Na;
+  S.Nb = Nb;
+  const std::vector<uint32_t>&ka = S.ka, &kb = S.kb;
+  const int64_t Da = int64_t(ka.size()), Db = int64_t(kb.size());
+  // shared memory of a block (complex amplitudes: the larger of the two)
+  const size_t smem = vqe::str_smem_bytes(int(std::min<int64_t>(Db, 65535)), 16);
+  if (Da * Db != int64_t(a->sector.size()) || Db > 8191 || smem > size_t(200) * 1024) return VQE_OK;  // not used
+  {
+    static std::mutex mu;
+    static size_t set_to = 0;
+    std::lock_guard<std::mutex> lk(mu);
+    if (smem > set_to) {
+      const cudaError_t ce = vqe::set_str_smem_limit(smem);
+      if (ce != cudaSuccess) return cuda_fail(ce, "string-driven H psi shared memory");
+      set_to = smem;
+    }
+  }
+  const uint32_t lo_mask = (1u << a->lo_bits) - 1u;
+  auto rank = [&](uint32_t k) { return a->rank_hi[k >> a->lo_bits] + a->rank_lo[k & lo_mask]; };
+  std::vector<uint32_t> perm(size_t(Da * Db));
+  parallel_ranges(Da, [&](int64_t lo, int64_t hi) {
+    for (int64_t i = lo; i < hi; ++i)
+      for (int64_t j = 0; j < Db; ++j) perm[size_t(i * Db + j)] = rank(ka[size_t(i)] | kb[size_t(j)]);
+  });
+  // the groups that can connect anything
+  const int G = int(h->groups.size());
+  std::vector<int> keep;
+  for (int g = 0; g < G; ++g) {
+    const uint32_t x = h->groups[g].x;
+    if ((pc32(x & even) & 1) == 0 && (pc32(x & odd) & 1) == 0) keep.push_back(g);
+  }
+  int rc;
+  if ((rc = upload_str(e, S.ka, &S.d_ka)) || (rc = upload_str(e, S.kb, &S.d_kb)) || (rc = upload_str(e, perm, &S.d_perm)))
+    return rc;
+  bool built = false;
+  if ((rc = build_buckets(h, S, keep, e, &e->str, &built)) != VQE_OK || !built) return rc;
+  if ((rc = build_tc(h, S, keep, e)) != VQE_OK) return rc;
+  std::vector<vqe::StrPlan> one(1, e->str);
   vqe::StrPlan* d_plan = nullptr;
-  if ((rc = up(one, &d_plan))) return rc;
+  if ((rc = upload_str(e, one, &d_plan))) return rc;
   e->d_str = d_plan;
   e->use_str = true;
   return VQE_OK;
@@ -982,12 +1335,20 @@ bool resident_fit(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, bool real, In
 
 struct WsLayout {
   size_t psi, lam, psi_am, lam_am, cs, epart, ctr, gpart, phi, total;
+  size_t dig, one_a, one_b, pexp, aexp, ade, bexp, bde, vi, vexp, vodd, vsum;  // tensor-core H psi (dig 0: none)
 };
 
 // Real sectors from this size keep the forward sweep's pair outputs for the
 // reverse sweep: psi and lambda (16 bytes per state together) no longer share
 // the L2, and the reverse step's gathers of both would miss it.
 constexpr size_t kKeepPhiMinStates = 6000000;
+
+size_t binomial(int n, int k) {
+  if (k < 0 || k > n) return 0;
+  double r = 1.0;
+  for (int i = 1; i <= k; ++i) r = r * (n - k + i) / i;
+  return size_t(r + 0.5);
+}
 
 WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   WsLayout L;
@@ -1005,6 +1366,30 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   const bool keep = !complex_amp && with_grad && a->sector.size() >= kKeepPhiMinStates;
   L.total = L.phi + (keep ? align256(size_t(a->pair_off.empty() ? 0 : a->pair_off.back()) * 16) : 0);
   if (!keep) L.phi = 0;
+  L.dig = 0;
+  if (!complex_amp && a->n_alpha >= 0 && int64_t(a->sector.size()) >= kTcMinStates) {
+    const int nb = a->n / 2, na = a->n - nb;  // beta and alpha qubits
+    const size_t Da = binomial(na, a->n_alpha), Db = binomial(nb, a->n_elec - a->n_alpha);
+    const size_t DaP = (Da + 63) / 64 * 64, DbP = (Db + 63) / 64 * 64, T = vqe::kTcDigits;
+    const size_t items = size_t(na) * size_t(na) + 1, R = size_t((nb * (nb + 1) / 2 + 127) / 128) * 128;
+    auto take = [&](size_t bytes) {
+      const size_t o = L.total;
+      L.total += align256(bytes);
+      return o;
+    };
+    L.dig = take(T * Da * DbP * 2);
+    L.one_a = take(T * Da * DaP * 2);
+    L.one_b = take(T * Db * DbP * 2);
+    L.pexp = take(Da * 4);
+    L.aexp = take(Da * 4);
+    L.ade = take(Da * 4);
+    L.bexp = take(Db * 4);
+    L.bde = take(Db * 4);
+    L.vi = take(2 * items * R * 8);
+    L.vexp = take(items * 4);
+    L.vodd = take(items * 4);
+    L.vsum = take(items * 8);
+  }
   return L;
 }
 
@@ -1019,6 +1404,21 @@ vqe::StreamBuffers buffers(void* ws, const WsLayout& L) {
   s.epart = reinterpret_cast<double*>(b + L.epart);
   s.gpart = reinterpret_cast<double*>(b + L.gpart);
   s.phi = L.phi ? reinterpret_cast<double2*>(b + L.phi) : nullptr;
+  std::memset(&s.tc, 0, sizeof(s.tc));
+  if (L.dig) {
+    s.tc.dig = reinterpret_cast<uint16_t*>(b + L.dig);
+    s.tc.one_a = reinterpret_cast<uint16_t*>(b + L.one_a);
+    s.tc.one_b = reinterpret_cast<uint16_t*>(b + L.one_b);
+    s.tc.pexp = reinterpret_cast<int*>(b + L.pexp);
+    s.tc.aexp = reinterpret_cast<int*>(b + L.aexp);
+    s.tc.ade = reinterpret_cast<int*>(b + L.ade);
+    s.tc.bexp = reinterpret_cast<int*>(b + L.bexp);
+    s.tc.bde = reinterpret_cast<int*>(b + L.bde);
+    s.tc.vi = reinterpret_cast<long long*>(b + L.vi);
+    s.tc.vexp = reinterpret_cast<int*>(b + L.vexp);
+    s.tc.vodd = reinterpret_cast<int*>(b + L.vodd);
+    s.tc.vsum = reinterpret_cast<double*>(b + L.vsum);
+  }
   return s;
 }
 
@@ -1106,6 +1506,10 @@ vqe::StreamPlan plan(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e) {
   p.use_ell = e->use_ell;
   p.use_str = e->use_str && !(g_flags & VQE_FLAG_NO_STRINGS);
   p.str = e->str;
+  p.use_tc = p.use_str && e->use_tc;
+  p.has_rest = e->has_rest;
+  p.tc = e->tc;
+  p.rest = e->rest;
   return p;
 }
 
@@ -1211,6 +1615,7 @@ int prepare_noalloc(vqe_hamiltonian_s* h, vqe_ansatz_s* a, bool with_grad, size_
   }
   *d = make_desc(h, a, e, 0);
   *sp = plan(a, e);
+  sp->use_tc = false;  // its operands do not fit the scratch
   sp->sweep = nullptr;  // one launch per gate: the sweep queues address the regular workspace layout
   // the string-driven H psi needs two more sector-sized vectors; when they do
   // not fit, the connectivity rows (if built) or the group scan serve instead

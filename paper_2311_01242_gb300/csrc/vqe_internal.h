@@ -84,6 +84,57 @@ struct StrPlan {
   const uint32_t* bob;
 };
 
+// Tensor-core H psi of a spin sector (vqe_tc.cu). Groups that flip one hop of each
+// spin, the occupation-dependent part of single hops and the mixed part of the
+// diagonal go through items and rows: an item is a directed alpha hop or an
+// occupied alpha qubit, a row an undirected beta hop or an occupied beta qubit.
+// Entry (Ia, k) of kj / kit is the k-th source of output alpha string Ia: source
+// string | sign << 31, and its item. Halfword Jb % 8 of dst[Jb / 8 * R + h] (R = 128 MT)
+// is the output beta string | sign << 13 | source holds the upper qubit << 14 | open << 15 (0: row
+// h is closed at Jb). vslot[item * R + h]: value slot | sign << 31 for a source
+// holding the lower and the upper qubit of the beta hop (-1: none). Everything that
+// moves one spin only is a row of that spin's matrix.
+constexpr int kTcDigits = 7;
+struct TcOneSpin {           // row r: entries [off[r], off[r + 1]), each the sum of its
+  int32_t n;                 // signed slots [soff[e], soff[e + 1]) at column col[e]
+  const int32_t* off;
+  const int32_t* col;
+  const int32_t* soff;
+  const uint32_t* slot;      // value slot | sign << 31
+};
+struct TcPlan {
+  int32_t Da, Db, DaP, DbP;  // DaP, DbP: rounded up to the tile width 64
+  int32_t K, KT, chunks;     // entries per output string, the same padded (64 chunks)
+  int32_t MT, items;
+  int32_t stages, sms;
+  const uint32_t* kj;
+  const uint16_t* kit;
+  const uint4* dst;
+  const int2* vslot;
+  TcOneSpin alpha, beta;
+};
+// its workspace: digits (fp16) of the signed source matrix and of the one-spin
+// matrices, with row exponents and sum bounds; the items' values
+struct TcScratch {
+  uint16_t* dig;             // [kTcDigits][Da][DbP]
+  uint16_t* one_a;           // [kTcDigits][Da][DaP]
+  uint16_t* one_b;           // [kTcDigits][Db][DbP]
+  int* pexp;                 // [Da]
+  int* aexp;                 // [Da], and its bounds
+  int* ade;
+  int* bexp;                 // [Db], and its bounds
+  int* bde;
+  long long* vi;             // [2][items][R]
+  int* vexp;                 // [items]
+  int* vodd;                 // [items]
+  double* vsum;              // [items]
+};
+int tc_stages(int DbP, size_t smem_limit);
+cudaError_t tc_set_smem_limit(size_t bytes);
+// lam_am (+)= the tensor-core part of H psi_am (both alpha-major, unsigned)
+cudaError_t tc_hpsi(const TcPlan& tc, const StrPlan& str, const TcScratch& sc, const double* vals,
+                    const double* psi_am, double* lam_am, bool add, cudaStream_t stream);
+
 struct InstDesc {
   // ansatz
   int32_t n, M;
@@ -265,6 +316,7 @@ struct StreamBuffers {
   // large real instances: the forward sweep's outputs {phi(k), phi(k ^ flip)} of
   // every pair, in pair order (null: the reverse sweep un-applies the gates to psi)
   double2* phi = nullptr;
+  TcScratch tc{};          // tensor-core H psi (used when the plan has use_tc)
   double2* cs;    // [M] (cos, sin)
   double* epart;  // [kMaxPartials]
   double* gpart;  // [M * kMaxPartials]
@@ -280,6 +332,10 @@ struct StreamPlan {
   bool use_ell;
   bool use_str;                  // string-driven H psi with `str`
   StrPlan str;
+  bool use_tc = false;           // real amplitudes: tc, and rest for the groups outside it
+  bool has_rest = false;
+  TcPlan tc;
+  StrPlan rest;
 };
 
 // Blocks of a streaming launch over `work` items (also the partial count).

@@ -905,12 +905,24 @@ cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuf
     T* lam_am = static_cast<T*>(b.lam_am);
     const size_t smem = str_smem_bytes(sp.str.Db, sizeof(T));
     k_perm_gather<REAL><<<grid, kStreamThreads, 0, stream>>>(sp.str.perm, d.D, psi, psi_am);
-    if (sp.str.Db >= kStrWideDb)
-      k_hpsi_str<REAL, true><<<str_blocks(sp.str.Da, sp.str.Db), kStrWarps * 32, smem, stream>>>(
-          sp.str, d.groups, d.emask, tv, psi_am, lam_am);
-    else
-      k_hpsi_str<REAL, false><<<str_blocks(sp.str.Da, sp.str.Db), kStrWarps * 32, smem, stream>>>(
-          sp.str, d.groups, d.emask, tv, psi_am, lam_am);
+    // with the tensor-core plan (and its workspace) the string-driven kernel sums
+    // only the groups outside it
+    const bool tc = REAL && sp.use_tc && b.tc.dig != nullptr;
+    const StrPlan& str = tc ? sp.rest : sp.str;
+    if (!tc || sp.has_rest) {
+      if (str.Db >= kStrWideDb)
+        k_hpsi_str<REAL, true><<<str_blocks(str.Da, str.Db), kStrWarps * 32, smem, stream>>>(
+            str, d.groups, d.emask, tv, psi_am, lam_am);
+      else
+        k_hpsi_str<REAL, false><<<str_blocks(str.Da, str.Db), kStrWarps * 32, smem, stream>>>(
+            str, d.groups, d.emask, tv, psi_am, lam_am);
+    }
+    if constexpr (REAL) {
+      if (tc) {
+        const cudaError_t e = tc_hpsi(sp.tc, sp.str, b.tc, d.vals, psi_am, lam_am, sp.has_rest, stream);
+        if (e != cudaSuccess) return e;
+      }
+    }
     k_perm_scatter<REAL><<<grid, kStreamThreads, 0, stream>>>(sp.str.perm, d.D, lam_am, lam);
     k_dot<REAL><<<grid, kStreamThreads, 0, stream>>>(psi, lam, d.D, b.epart);
   } else if (sp.use_ell) {
