@@ -396,6 +396,15 @@ struct PersistQueue {
 struct StreamBatch {
   std::vector<int> slots;                 // batch index of each persistent slot
   std::vector<int> big;                   // batch indices evaluated one by one (too large for a slot)
+  std::vector<int> mid;                   // batch indices swept in cluster shared memory
+  std::vector<size_t> mid_off;            // their workspace layouts
+  std::vector<vqe::SweepClass> classes;   // by cluster size
+  vqe::SweepInst* d_sweep = nullptr;      // class by class
+  vqe::TcInst* d_tc = nullptr;
+  int2* d_tiles = nullptr;
+  int2* d_rows = nullptr;
+  vqe::TcBatch tcb;
+  int mid_ctas = 0;
   std::vector<InstDesc> descs;            // per slot
   std::vector<vqe::PSlot> pslots;
   InstDesc* d_desc = nullptr;
@@ -410,6 +419,10 @@ struct StreamBatch {
   int probe_task = -1;
   int last_queue = 1;                     // queue of the last launch (for status messages)
   ~StreamBatch() {
+    dfree(d_sweep);
+    dfree(d_tc);
+    dfree(d_tiles);
+    dfree(d_rows);
     dfree(d_desc);
     dfree(d_slots);
   }
@@ -717,10 +730,11 @@ int build_buckets(vqe_hamiltonian_t h, const Strings& S, std::vector<int> keep, 
   return VQE_OK;
 }
 
-// Sectors from this size on evaluate their hop x hop groups on the tensor cores.
-// (Smaller ones also run inside the batch's persistent launch, whose results equal
-// the single calls' bit for bit.)
-constexpr int64_t kTcMinStates = int64_t(vqe::kMaxPartials) * vqe::kStreamThreads + 1;
+// Sectors from this size on run H psi on the tensor cores. Up to kMidStates, where a
+// batch's persistent launch would evaluate them with other kernels than a single
+// call (whose results it equals bit for bit), only without groups outside that form.
+constexpr int64_t kTcMinStates = 256;
+constexpr int64_t kMidStates = int64_t(vqe::kMaxPartials) * vqe::kStreamThreads;
 
 // How the tensor-core H psi takes a group. Amplitudes are multiplied by s(Ia, Ib) =
 // (-1)^{alpha electrons above beta ones}; a group is taken when its sign then
@@ -932,7 +946,7 @@ int build_tc(vqe_hamiltonian_t h, const Strings& S, const std::vector<int>& keep
       case TcKind::kNone: rest.push_back(gi); break;
     }
   }
-  if (rest.size() == keep.size()) return VQE_OK;
+  if (rest.size() == keep.size() || (!rest.empty() && Da * Db <= kMidStates)) return VQE_OK;
   // sources of every output alpha string
   std::vector<std::vector<std::pair<uint32_t, uint16_t>>> src(static_cast<size_t>(Da));
   parallel_ranges(Da, [&](int64_t lo, int64_t hi) {
@@ -1011,7 +1025,8 @@ int build_tc(vqe_hamiltonian_t h, const Strings& S, const std::vector<int>& keep
   T.kit = d_kit;
   T.dst = d_dst;
   T.vslot = d_vslot;
-  const cudaError_t ce = vqe::tc_set_smem_limit(size_t(optin));
+  cudaError_t ce = vqe::tc_set_smem_limit(size_t(optin));
+  if (ce == cudaSuccess) ce = vqe::sweep_set_limits(size_t(optin));
   if (ce != cudaSuccess) return cuda_fail(ce, "tensor-core H psi shared memory");
   e->tc = T;
   e->use_tc = true;
@@ -1335,7 +1350,9 @@ bool resident_fit(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, bool real, In
 
 struct WsLayout {
   size_t psi, lam, psi_am, lam_am, cs, epart, ctr, gpart, phi, total;
-  size_t dig, one_a, one_b, pexp, aexp, ade, bexp, bde, vi, vexp, vodd, vsum;  // tensor-core H psi (dig 0: none)
+  bool has_tc;
+  vqe::TcOffsets tc;  // tensor-core H psi
+  size_t sw_phi, sw_gacc, sw_dot;  // sweeps in cluster shared memory
 };
 
 // Real sectors from this size keep the forward sweep's pair outputs for the
@@ -1348,6 +1365,16 @@ size_t binomial(int n, int k) {
   double r = 1.0;
   for (int i = 1; i <= k; ++i) r = r * (n - k + i) / i;
   return size_t(r + 0.5);
+}
+
+// Whether the gate sweeps of this ansatz can run in cluster shared memory. Beyond 2^17
+// states a gate's pairs take longer on sixteen SMs than a launch over all of them (22
+// qubits: 4.2 against 3.2 us).
+constexpr int64_t kSweepStates = int64_t(1) << 17;
+bool mid_ansatz(vqe_ansatz_t a) {
+  const int64_t D = int64_t(a->sector.size());
+  return a->n_alpha >= 0 && D >= kTcMinStates && D <= kSweepStates && a->M <= 2048 &&
+         int64_t(a->pairs.size()) < (int64_t(1) << 30);
 }
 
 WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
@@ -1366,8 +1393,9 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   const bool keep = !complex_amp && with_grad && a->sector.size() >= kKeepPhiMinStates;
   L.total = L.phi + (keep ? align256(size_t(a->pair_off.empty() ? 0 : a->pair_off.back()) * 16) : 0);
   if (!keep) L.phi = 0;
-  L.dig = 0;
-  if (!complex_amp && a->n_alpha >= 0 && int64_t(a->sector.size()) >= kTcMinStates) {
+  std::memset(&L.tc, 0, sizeof(L.tc));
+  L.has_tc = !complex_amp && a->n_alpha >= 0 && int64_t(a->sector.size()) >= kTcMinStates;
+  if (L.has_tc) {
     const int nb = a->n / 2, na = a->n - nb;  // beta and alpha qubits
     const size_t Da = binomial(na, a->n_alpha), Db = binomial(nb, a->n_elec - a->n_alpha);
     const size_t DaP = (Da + 63) / 64 * 64, DbP = (Db + 63) / 64 * 64, T = vqe::kTcDigits;
@@ -1375,20 +1403,29 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
     auto take = [&](size_t bytes) {
       const size_t o = L.total;
       L.total += align256(bytes);
-      return o;
+      return int64_t(o);
     };
-    L.dig = take(T * Da * DbP * 2);
-    L.one_a = take(T * Da * DaP * 2);
-    L.one_b = take(T * Db * DbP * 2);
-    L.pexp = take(Da * 4);
-    L.aexp = take(Da * 4);
-    L.ade = take(Da * 4);
-    L.bexp = take(Db * 4);
-    L.bde = take(Db * 4);
-    L.vi = take(2 * items * R * 8);
-    L.vexp = take(items * 4);
-    L.vodd = take(items * 4);
-    L.vsum = take(items * 8);
+    L.tc.dig = take(T * Da * DbP * 2);
+    L.tc.one_a = take(T * Da * DaP * 2);
+    L.tc.one_b = take(T * Db * DbP * 2);
+    L.tc.pexp = take(Da * 4);
+    L.tc.aexp = take(Da * 4);
+    L.tc.ade = take(Da * 4);
+    L.tc.bexp = take(Db * 4);
+    L.tc.bde = take(Db * 4);
+    L.tc.vi = take(2 * items * R * 8);
+    L.tc.vexp = take(items * 4);
+    L.tc.vodd = take(items * 4);
+    L.tc.vsum = take(items * 8);
+    L.tc.psi_am = int64_t(L.psi_am);
+    L.tc.lam_am = int64_t(L.lam_am);
+  }
+  L.sw_phi = L.sw_gacc = L.sw_dot = 0;
+  if (L.has_tc && mid_ansatz(a)) {
+    L.sw_gacc = L.total;
+    L.sw_dot = L.sw_gacc + align256(size_t(std::max(a->M, 1)) * 8);
+    L.sw_phi = L.sw_dot + align256(size_t(2 * vqe::kSweepDots) * 8);
+    L.total = L.sw_phi + (with_grad ? align256(std::max<size_t>(a->pairs.size(), 1) * 16) : 0);
   }
   return L;
 }
@@ -1404,21 +1441,9 @@ vqe::StreamBuffers buffers(void* ws, const WsLayout& L) {
   s.epart = reinterpret_cast<double*>(b + L.epart);
   s.gpart = reinterpret_cast<double*>(b + L.gpart);
   s.phi = L.phi ? reinterpret_cast<double2*>(b + L.phi) : nullptr;
-  std::memset(&s.tc, 0, sizeof(s.tc));
-  if (L.dig) {
-    s.tc.dig = reinterpret_cast<uint16_t*>(b + L.dig);
-    s.tc.one_a = reinterpret_cast<uint16_t*>(b + L.one_a);
-    s.tc.one_b = reinterpret_cast<uint16_t*>(b + L.one_b);
-    s.tc.pexp = reinterpret_cast<int*>(b + L.pexp);
-    s.tc.aexp = reinterpret_cast<int*>(b + L.aexp);
-    s.tc.ade = reinterpret_cast<int*>(b + L.ade);
-    s.tc.bexp = reinterpret_cast<int*>(b + L.bexp);
-    s.tc.bde = reinterpret_cast<int*>(b + L.bde);
-    s.tc.vi = reinterpret_cast<long long*>(b + L.vi);
-    s.tc.vexp = reinterpret_cast<int*>(b + L.vexp);
-    s.tc.vodd = reinterpret_cast<int*>(b + L.vodd);
-    s.tc.vsum = reinterpret_cast<double*>(b + L.vsum);
-  }
+  s.base = b;
+  s.has_tc = L.has_tc;
+  s.tc = L.tc;
   return s;
 }
 
@@ -1566,6 +1591,114 @@ cudaError_t stream_eval(const InstDesc& d, const vqe::StreamPlan& sp, const vqe:
   return vqe::stream_energy_grad(d, sp, b, real, with_grad, theta, energy, grad, stream);
 }
 
+// Cluster sizes of the gate sweeps: the smallest that holds the state, then larger
+// ones while a gate's estimated clocks fall (its pairs at 6.7 multiplies per clock
+// and SM, ten per pair over both sweeps, plus the chain of both gates' loads, stores
+// and barriers) and CTAs are free.
+struct SweepShape {
+  int c = 0, shift = 0, threads = 0;
+  size_t smem = 0;
+};
+// Threads per CTA: what every warp does per gate costs issue slots, so few where a
+// CTA's share of a gate is small.
+int sweep_threads(vqe_ansatz_t a, int c) {
+  const double share = a->M > 0 ? double(a->pairs.size()) / a->M / c : 0.0;
+  return share <= 192.0 ? 128 : share <= 384.0 ? 256 : 512;
+}
+bool sweep_shape(vqe_ansatz_t a, int c, size_t optin, SweepShape* out) {
+  const int64_t D = int64_t(a->sector.size());
+  int shift = 0;
+  while ((int64_t(c) << shift) < D) ++shift;
+  out->c = c;
+  out->shift = shift;
+  out->threads = sweep_threads(a, c);
+  out->smem = vqe::sweep_smem(a->M, c, shift, D, out->threads);
+  return out->smem + 1024 <= optin && (c == 1 || shift <= vqe::kSweepMaxShift) && (c <= 8 || vqe::sweep_wide_clusters());
+}
+double sweep_clocks(vqe_ansatz_t a, int c) {
+  const double pairs = a->M > 0 ? double(a->pairs.size()) / a->M : 0.0;
+  return a->M * ((c == 1 ? 500.0 : 1400.0) + 10.0 / 6.7 * pairs / c);
+}
+bool smallest_shape(vqe_ansatz_t a, size_t optin, SweepShape* s) {
+  for (int c = 1; c <= 16; c *= 2)
+    if (sweep_shape(a, c, optin, s)) return true;
+  return false;
+}
+int device_limits(size_t* optin, int* sms) {
+  int dev = 0, o = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&o, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  *optin = size_t(o);
+  return e == cudaSuccess ? VQE_OK : cuda_fail(e, "device attributes");
+}
+
+// Real instances whose gate sweeps run in cluster shared memory and whose H psi is
+// wholly on the tensor cores.
+bool mid_flags() {
+  return use_real() && !(g_flags & (VQE_FLAG_FP64_SWEEPS | VQE_FLAG_NO_STRINGS));
+}
+bool mid_fits(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e) {
+  SweepShape s;
+  size_t optin = 0;
+  int sms = 0;
+  return e->use_tc && !e->has_rest && mid_ansatz(a) && device_limits(&optin, &sms) == VQE_OK &&
+         smallest_shape(a, optin, &s);
+}
+
+vqe::SweepInst sweep_inst(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, const InstDesc& d, const WsLayout& L,
+                          size_t base, const SweepShape& s) {
+  vqe::SweepInst I;
+  std::memset(&I, 0, sizeof(I));
+  I.M = a->M;
+  I.D = int32_t(a->sector.size());
+  I.shift = s.shift;
+  I.hf_rank = d.hf_rank;
+  I.pair_off = d.pair_off;
+  I.rpairs = d.rpairs;
+  I.perm = e->str.perm;
+  I.inst = d.inst;
+  I.psi_am = int64_t(base + L.psi_am);
+  I.lam_am = int64_t(base + L.lam_am);
+  I.phi = int64_t(base + L.sw_phi);
+  I.gacc = int64_t(base + L.sw_gacc);
+  I.dot = int64_t(base + L.sw_dot);
+  return I;
+}
+
+vqe::TcInst tc_inst(vqe_hamiltonian_t h, const vqe_hamiltonian_s::Ell* e, const WsLayout& L, size_t base) {
+  vqe::TcInst I{e->tc, L.tc, e->str.ka, e->str.kb, h->d_vals};
+  int64_t* o = reinterpret_cast<int64_t*>(&I.off);
+  for (size_t i = 0; i < sizeof(I.off) / sizeof(int64_t); ++i) o[i] += int64_t(base);
+  return I;
+}
+
+int run_mid(vqe_hamiltonian_t h, vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, const InstDesc& d,
+            const double* theta, double* energy, double* grad, char* ws, const WsLayout& L, cudaStream_t stream) {
+  size_t optin = 0;
+  int sms = 0;
+  int rc = device_limits(&optin, &sms);
+  if (rc) return rc;
+  SweepShape s;
+  if (!smallest_shape(a, optin, &s)) return fail(VQE_ERR_UNSUPPORTED, "sweeps do not fit shared memory");
+  for (int c = 2 * s.c; c <= 16; c *= 2) {
+    SweepShape t;
+    if (sweep_clocks(a, c) < sweep_clocks(a, s.c) && sweep_shape(a, c, optin, &t)) s = t;
+  }
+  InstDesc d0 = d;
+  d0.inst = 0;
+  const vqe::SweepInst I = sweep_inst(a, e, d0, L, 0, s);
+  const vqe::SweepClass k{nullptr, 1, s.c, s.threads, false, s.smem};
+  const vqe::SweepCtl ctl{nullptr, nullptr, 0, -1, 0, 0};
+  const vqe::TcInst T = tc_inst(h, e, L, 0);
+  cudaError_t ce = vqe::sweep_forward(k, &I, ws, theta, 0, grad != nullptr, ctl, stream);
+  if (ce == cudaSuccess) ce = vqe::tc_hpsi(vqe::tc_single(e->tc), &T, ws, false, stream);
+  if (ce == cudaSuccess) ce = vqe::sweep_dots(nullptr, &I, 1, ws, stream);
+  if (ce == cudaSuccess && grad) ce = vqe::sweep_reverse(k, &I, ws, theta, 0, ctl, stream);
+  if (ce == cudaSuccess) ce = vqe::sweep_final(nullptr, &I, 1, ws, ctl, energy, grad, 0, stream);
+  return ce == cudaSuccess ? VQE_OK : cuda_fail(ce, "cluster sweeps launch");
+}
+
 int run_single(vqe_hamiltonian_t h, vqe_ansatz_t a, const double* theta, double* energy, double* grad,
                void* ws, size_t ws_bytes, cudaStream_t stream, bool with_grad) {
   int rc = check_pair(h, a);
@@ -1586,6 +1719,8 @@ int run_single(vqe_hamiltonian_t h, vqe_ansatz_t a, const double* theta, double*
   }
   const WsLayout L = ws_layout(a, !real, with_grad);
   if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
+  if (mid_flags() && mid_fits(a, e))
+    return run_mid(h, a, e, d, theta, energy, with_grad ? grad : nullptr, static_cast<char*>(ws), L, stream);
   cudaError_t ce = stream_eval(d, plan(a, e), buffers(ws, L), real, with_grad, theta, energy, grad, stream);
   if (ce != cudaSuccess) return cuda_fail(ce, "streaming launch");
   return VQE_OK;
@@ -2666,17 +2801,130 @@ static int persist_grid(const StreamBatch& sb, int* grid) {
   return VQE_OK;
 }
 
+// The batch's instances swept in cluster shared memory: workspace layouts after the
+// persistent slots', cluster sizes, and the tensor-core work lists (costly instances
+// first).
+static int build_mid_batch(vqe_batch_s* B) {
+  StreamBatch& sb = B->sb;
+  const int n = int(sb.mid.size());
+  if (n == 0) return VQE_OK;
+  size_t optin = 0;
+  int sms = 0, rc;
+  if ((rc = device_limits(&optin, &sms))) return rc;
+  std::vector<SweepShape> shape(static_cast<size_t>(n));
+  int total = 0;
+  for (int i = 0; i < n; ++i) {
+    smallest_shape(B->ans[sb.mid[size_t(i)]], optin, &shape[size_t(i)]);
+    total += shape[size_t(i)].c;
+  }
+  // widen the slowest while that helps it and every cluster still runs at once
+  std::vector<char> fixed(static_cast<size_t>(n), 0);
+  for (;;) {
+    int top = -1;
+    double most = -1.0;
+    for (int i = 0; i < n; ++i) {
+      const double t = sweep_clocks(B->ans[sb.mid[size_t(i)]], shape[size_t(i)].c);
+      if (!fixed[size_t(i)] && t > most) {
+        most = t;
+        top = i;
+      }
+    }
+    if (top < 0) break;
+    vqe_ansatz_t a = B->ans[sb.mid[size_t(top)]];
+    SweepShape& s = shape[size_t(top)];
+    SweepShape t;
+    if (s.c < 16 && total + s.c <= sms && sweep_clocks(a, 2 * s.c) < sweep_clocks(a, s.c) &&
+        sweep_shape(a, 2 * s.c, optin, &t)) {
+      total += s.c;
+      s = t;
+    } else {
+      fixed[size_t(top)] = 1;
+    }
+  }
+  sb.mid_ctas = total;
+  std::vector<vqe::SweepInst> sweep;
+  std::vector<vqe::TcInst> tcs;
+  std::vector<std::pair<int64_t, int>> order;
+  size_t off = sb.persist_bytes;
+  std::vector<size_t> first;
+  for (int i = 0; i < n; ++i) {
+    const int b = sb.mid[size_t(i)];
+    const auto* e = get_ell(B->hams[b], B->ans[b], &rc);
+    if (!e) return rc;
+    const WsLayout L = ws_layout(B->ans[b], false, true);
+    sb.mid_off.push_back(off);
+    tcs.push_back(tc_inst(B->hams[b], e, L, off));
+    order.push_back({-int64_t(e->tc.DbP) * e->tc.K, i});
+    const vqe::TcPlan& T = e->tc;
+    vqe::TcBatch& t = sb.tcb;
+    t.items = std::max(t.items, int(T.items));
+    t.Da = std::max(t.Da, int(T.Da));
+    t.Db = std::max(t.Db, int(T.Db));
+    t.DaP = std::max(t.DaP, int(T.DaP));
+    t.DbP = std::max(t.DbP, int(T.DbP));
+    t.stages = i ? std::min(t.stages, int(T.stages)) : int(T.stages);
+    off += L.total;
+  }
+  for (int c = 16; c >= 1; c /= 2) {
+    vqe::SweepClass k{nullptr, 0, c, 0, !sb.classes.empty(), 0};
+    first.push_back(sweep.size());
+    for (int i = 0; i < n; ++i) {
+      if (shape[size_t(i)].c != c) continue;
+      const int b = sb.mid[size_t(i)];
+      const auto* e = get_ell(B->hams[b], B->ans[b], &rc);
+      if (!e) return rc;
+      sweep.push_back(sweep_inst(B->ans[b], e, B->descs[b], ws_layout(B->ans[b], false, true), sb.mid_off[size_t(i)],
+                                 shape[size_t(i)]));
+      sweep.back().task = int32_t(sweep.size()) - 1;
+      k.threads = std::max(k.threads, shape[size_t(i)].threads);
+      ++k.n;
+    }
+    for (size_t j = first.back(); j < sweep.size(); ++j)
+      k.smem = std::max(k.smem, vqe::sweep_smem(sweep[j].M, c, sweep[j].shift, sweep[j].D, k.threads));
+    if (k.n > 0)
+      sb.classes.push_back(k);
+    else
+      first.pop_back();
+  }
+  std::sort(order.begin(), order.end());
+  std::vector<int2> tiles, rows;
+  for (const auto& o : order) {
+    const vqe::TcPlan& T = tcs[size_t(o.second)].tc;
+    for (int t = 0; t < vqe::tc_tiles(T); ++t) tiles.push_back(make_int2(o.second, t));
+    for (int r = 0; r < T.Da; ++r) rows.push_back(make_int2(o.second, r));
+  }
+  if ((rc = upload(sweep, &sb.d_sweep)) || (rc = upload(tcs, &sb.d_tc)) || (rc = upload(tiles, &sb.d_tiles)) ||
+      (rc = upload(rows, &sb.d_rows)))
+    return rc;
+  for (size_t k = 0; k < sb.classes.size(); ++k) sb.classes[k].insts = sb.d_sweep + first[k];
+  vqe::TcBatch& t = sb.tcb;
+  t.insts = sb.d_tc;
+  t.tiles = sb.d_tiles;
+  t.rows = sb.d_rows;
+  t.n = n;
+  t.n_tiles = int(tiles.size());
+  t.n_rows = int(rows.size());
+  t.sms = sms;
+  sb.persist_bytes = off;
+  return VQE_OK;
+}
+
 static int build_stream_batch(vqe_batch_s* B) {
   StreamBatch& sb = B->sb;
   for (int i : B->streaming[0]) {
-    if (slot_fits(B->ans[i]))
+    int rc = VQE_OK;
+    const auto* e = get_ell(B->hams[i], B->ans[i], &rc);
+    if (!e) return rc;
+    if (mid_fits(B->ans[i], e))
+      sb.mid.push_back(i);
+    else if (slot_fits(B->ans[i]) && !e->use_tc)
       sb.slots.push_back(i);
     else
       sb.big.push_back(i);
   }
   for (int i : sb.big) sb.big_bytes = std::max(sb.big_bytes, ws_layout(B->ans[i], false, true).total);
   const int n = int(sb.slots.size());
-  if (n == 0) return VQE_OK;
+  if (n == 0 && sb.mid.empty()) return VQE_OK;
   size_t off = 0;
   for (int s = 0; s < n; ++s) {
     const int i = sb.slots[s];
@@ -2711,8 +2959,10 @@ static int build_stream_batch(vqe_batch_s* B) {
     sb.pslots.push_back(ps);
   }
   sb.counters_off = off;
-  sb.persist_bytes = off + align256(size_t(n + 2) * sizeof(int));
+  sb.persist_bytes = off + align256(size_t(n + 3) * sizeof(int));  // and one that stays zero
   int rc;
+  if ((rc = build_mid_batch(B))) return rc;
+  if (n == 0) return VQE_OK;
   if ((rc = upload(sb.descs, &sb.d_desc))) return rc;
   if ((rc = upload(sb.pslots, &sb.d_slots))) return rc;
   if ((rc = persist_grid(sb, &sb.grid))) return rc;
@@ -2762,7 +3012,7 @@ int32_t vqe_batch_max_params(vqe_batch_t b) { return b ? b->max_params : 0; }
 // Streamed instances run one by one (stream_energy_grad) in complex mode, under
 // VQE_FLAG_NO_STRINGS, and for instances too large for a persistent slot.
 static bool persistent_mode(vqe_batch_t b, bool real) {
-  return real && !(g_flags & VQE_FLAG_NO_STRINGS) && !b->sb.slots.empty();
+  return real && !(g_flags & VQE_FLAG_NO_STRINGS) && !(b->sb.slots.empty() && b->sb.mid.empty());
 }
 
 size_t vqe_batch_workspace_bytes(vqe_batch_t b, int with_grad) {
@@ -2819,24 +3069,53 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
     const StreamBatch& sb = b->sb;
     const size_t need = vqe_batch_workspace_bytes(b, with_grad);
     if ((rc = check_ws(ws, ws_bytes, need))) return rc;
-    const PersistQueue& Q = *sb.q[with_grad ? 1 : 0];
     b->sb.last_queue = with_grad ? 1 : 0;
-    vqe::PersistDev pd;
-    pd.desc = sb.d_desc;
-    pd.slots = sb.d_slots;
-    pd.tasks = Q.d_tasks;
-    pd.n_tasks = int32_t(Q.tasks.size());
-    pd.n = int32_t(sb.slots.size());
-    pd.ws = static_cast<char*>(ws);
-    pd.counters = reinterpret_cast<int*>(static_cast<char*>(ws) + sb.counters_off);
-    pd.budget_ns = sb.budget_ns;
-    pd.probe_task = sb.probe_task;
-    pd.pad = 0;
-    if ((rc = ensure_persist_smem(sb.smem))) return rc;
-    cudaError_t ce = vqe::batch_persistent_run(pd, sb.grid, sb.smem, Q.d_finals, int(Q.finals.size()),
-                                               Q.n_grad_rows, theta, ld_theta, energies,
-                                               with_grad ? grads : nullptr, ld_grad, stream);
-    if (ce != cudaSuccess) return cuda_fail(ce, "persistent batch launch");
+    int* counters = reinterpret_cast<int*>(static_cast<char*>(ws) + sb.counters_off);
+    const int n_slots = int(sb.slots.size());
+    int queued = 0;
+    cudaError_t ce = cudaMemsetAsync(counters, 0, size_t(n_slots + 3) * sizeof(int), stream);
+    if (ce != cudaSuccess) return cuda_fail(ce, "batch counters");
+    if (n_slots > 0) {
+      const PersistQueue& Q = *sb.q[with_grad ? 1 : 0];
+      vqe::PersistDev pd;
+      pd.desc = sb.d_desc;
+      pd.slots = sb.d_slots;
+      pd.tasks = Q.d_tasks;
+      pd.n_tasks = queued = int32_t(Q.tasks.size());
+      pd.n = int32_t(n_slots);
+      pd.ws = static_cast<char*>(ws);
+      pd.counters = counters;
+      pd.budget_ns = sb.budget_ns;
+      pd.probe_task = sb.probe_task;
+      pd.pad = 0;
+      if ((rc = ensure_persist_smem(sb.smem))) return rc;
+      ce = vqe::batch_persistent_run(pd, sb.grid, sb.smem, Q.d_finals, int(Q.finals.size()), Q.n_grad_rows, theta,
+                                     ld_theta, energies, with_grad ? grads : nullptr, ld_grad, stream);
+      if (ce != cudaSuccess) return cuda_fail(ce, "persistent batch launch");
+    }
+    if (!sb.mid.empty() && mid_flags()) {
+      char* w = static_cast<char*>(ws);
+      const int n = int(sb.mid.size());
+      const vqe::SweepCtl ctl{counters + n_slots + 1, counters + n_slots + 2, sb.budget_ns, sb.probe_task, queued, n};
+      ce = cudaSuccess;
+      for (const auto& k : sb.classes)
+        if (ce == cudaSuccess) ce = vqe::sweep_forward(k, nullptr, w, theta, ld_theta, with_grad, ctl, stream);
+      if (ce == cudaSuccess) ce = vqe::tc_hpsi(sb.tcb, nullptr, w, false, stream);
+      if (ce == cudaSuccess) ce = vqe::sweep_dots(sb.d_sweep, nullptr, n, w, stream);
+      if (with_grad)
+        for (const auto& k : sb.classes)
+          if (ce == cudaSuccess) ce = vqe::sweep_reverse(k, nullptr, w, theta, ld_theta, ctl, stream);
+      if (ce == cudaSuccess)
+        ce = vqe::sweep_final(sb.d_sweep, nullptr, n, w, ctl, energies, with_grad ? grads : nullptr, ld_grad, stream);
+      if (ce != cudaSuccess) return cuda_fail(ce, "batched cluster sweeps launch");
+    } else {
+      for (size_t k = 0; k < sb.mid.size(); ++k) {
+        const size_t off = sb.mid_off[k];
+        rc = run_one_by_one(b, std::vector<int>(1, sb.mid[k]), true, theta, ld_theta, energies, grads, ld_grad,
+                            static_cast<char*>(ws) + off, sb.persist_bytes - off, stream);
+        if (rc) return rc;
+      }
+    }
     if (!sb.big.empty())
       return run_one_by_one(b, sb.big, true, theta, ld_theta, energies, grads, ld_grad,
                             static_cast<char*>(ws) + sb.persist_bytes, ws_bytes - sb.persist_bytes, stream);
@@ -2979,9 +3258,12 @@ int vqe_batch_set_tuning(vqe_batch_t b, int ctas_per_sm, int gate_chunk, int swe
     return fail(VQE_ERR_INVALID_ARG, "sweep_threads: a multiple of 32 in [32, 512], or 0 to keep");
   ++b->tuning_version;  // launch shapes are captured in the host-call graph
   StreamBatch& sb = b->sb;
-  if (!sb.slots.empty() && (ctas_per_sm != sb.ctas_per_sm || (gate_chunk && gate_chunk != sb.gate_chunk))) {
+  const bool changed = ctas_per_sm != sb.ctas_per_sm || (gate_chunk && gate_chunk != sb.gate_chunk);
+  if (changed && !(sb.slots.empty() && sb.mid.empty())) {
     sb.ctas_per_sm = ctas_per_sm;
     if (gate_chunk) sb.gate_chunk = gate_chunk;
+  }
+  if (changed && !sb.slots.empty()) {  // (cluster sweeps have no such choice)
     int rc = persist_grid(sb, &sb.grid);
     if (rc == VQE_OK) rc = build_queues(b);
     if (rc) return rc;
@@ -3003,8 +3285,8 @@ int vqe_batch_get_tuning(vqe_batch_t b, int* ctas_per_sm, int* gate_chunk, int* 
   if (!b) return fail(VQE_ERR_INVALID_ARG, "NULL batch");
   if (ctas_per_sm) *ctas_per_sm = b->sb.ctas_per_sm;
   if (gate_chunk) *gate_chunk = b->sb.gate_chunk;
-  if (grid) *grid = b->sb.slots.empty() ? 0 : b->sb.grid;
-  if (n_tasks) *n_tasks = b->sb.q[1] ? int64_t(b->sb.q[1]->tasks.size()) : 0;
+  if (grid) *grid = b->sb.slots.empty() ? b->sb.mid_ctas : b->sb.grid;
+  if (n_tasks) *n_tasks = (b->sb.q[1] ? int64_t(b->sb.q[1]->tasks.size()) : 0) + 2 * int64_t(b->sb.mid.size());
   return VQE_OK;
 }
 
@@ -3022,7 +3304,7 @@ int vqe_batch_set_wait(vqe_batch_t b, int64_t budget_ns, int32_t probe_task) {
 int vqe_batch_status(vqe_batch_t b, const void* ws, size_t ws_bytes, vqe_stream_t stream) {
   if (!b) return fail(VQE_ERR_INVALID_ARG, "NULL batch");
   const StreamBatch& sb = b->sb;
-  if (sb.slots.empty()) return VQE_OK;
+  if (sb.slots.empty() && sb.mid.empty()) return VQE_OK;
   if (!ws || ws_bytes < sb.persist_bytes) return fail(VQE_ERR_WORKSPACE, "workspace smaller than the batch's");
   int status = 0;
   cudaError_t ce = cudaMemcpyAsync(&status, static_cast<const char*>(ws) + sb.counters_off + (sb.slots.size() + 1) * sizeof(int),

@@ -129,11 +129,45 @@ struct TcScratch {
   int* vodd;                 // [items]
   double* vsum;              // [items]
 };
+struct TcOffsets {           // the same as byte offsets from the workspace's start, and the
+  int64_t dig, one_a, one_b, pexp, aexp, ade, bexp, bde, vi, vexp, vodd, vsum;
+  int64_t psi_am, lam_am;    // alpha-major source and result (unsigned, FP64)
+};
+struct TcInst {
+  TcPlan tc;
+  TcOffsets off;
+  const uint32_t* ka;        // [Da], [Db] strings
+  const uint32_t* kb;
+  const double* vals;
+};
+// What a launch over one instance (insts unused) or a batch needs: the largest
+// sizes, and for a batch the (instance, tile) and (instance, output string) lists.
+struct TcBatch {
+  const TcInst* insts = nullptr;
+  const int2* tiles = nullptr;
+  const int2* rows = nullptr;
+  int n = 1, n_tiles = 0, n_rows = 0;
+  int items = 0, Da = 0, Db = 0, DaP = 0, DbP = 0;
+  int stages = 0, sms = 0;
+};
 int tc_stages(int DbP, size_t smem_limit);
+int tc_tiles(const TcPlan& tc);
 cudaError_t tc_set_smem_limit(size_t bytes);
-// lam_am (+)= the tensor-core part of H psi_am (both alpha-major, unsigned)
-cudaError_t tc_hpsi(const TcPlan& tc, const StrPlan& str, const TcScratch& sc, const double* vals,
-                    const double* psi_am, double* lam_am, bool add, cudaStream_t stream);
+// lam_am (+)= the tensor-core part of H psi_am, for *one or every instance of B
+cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, cudaStream_t stream);
+inline TcBatch tc_single(const TcPlan& tc) {
+  TcBatch b;
+  b.n_tiles = tc_tiles(tc);
+  b.n_rows = tc.Da;
+  b.items = tc.items;
+  b.Da = tc.Da;
+  b.Db = tc.Db;
+  b.DaP = tc.DaP;
+  b.DbP = tc.DbP;
+  b.stages = tc.stages;
+  b.sms = tc.sms;
+  return b;
+}
 
 struct InstDesc {
   // ansatz
@@ -316,11 +350,48 @@ struct StreamBuffers {
   // large real instances: the forward sweep's outputs {phi(k), phi(k ^ flip)} of
   // every pair, in pair order (null: the reverse sweep un-applies the gates to psi)
   double2* phi = nullptr;
-  TcScratch tc{};          // tensor-core H psi (used when the plan has use_tc)
+  char* base = nullptr;    // the workspace
+  bool has_tc = false;     // ... has the tensor-core H psi's part, at
+  TcOffsets tc{};
   double2* cs;    // [M] (cos, sin)
   double* epart;  // [kMaxPartials]
   double* gpart;  // [M * kMaxPartials]
 };
+
+// Gate sweeps of mid-size real instances in cluster shared memory (vqe_sweep.cu).
+constexpr int kSweepDots = 32;       // partial sums of psi . lambda and lambda . lambda
+constexpr int kSweepMaxShift = 14;   // at most 2^14 amplitudes per CTA of a cluster
+struct SweepInst {
+  int32_t M, D, shift, hf_rank;      // amplitude r lives in CTA r >> shift (one CTA: unused)
+  const int64_t* pair_off;
+  const uint2* rpairs;
+  const uint32_t* perm;              // alpha-major index -> rank
+  int64_t inst;                      // row in the caller's arrays
+  int32_t task, pad;                 // number among the batch's sweeps
+  int64_t psi_am, lam_am, phi, gacc, dot;  // byte offsets in the workspace
+};
+struct SweepClass {                  // instances of one cluster size
+  const SweepInst* insts;
+  int n, c, threads;
+  bool follows;                      // launched beside the class before it
+  size_t smem;
+};
+struct SweepCtl {                    // a batch's wait check (single calls: status null, probe -1)
+  int* status;
+  const int* never;
+  long long budget_ns;
+  int probe, task0, n;               // forward sweeps are tasks task0 + i, reverse ones task0 + n + i
+};
+size_t sweep_smem(int M, int c, int shift, int64_t D, int threads);
+cudaError_t sweep_set_limits(size_t optin);
+bool sweep_wide_clusters();          // whether clusters of 16 can be resident
+cudaError_t sweep_forward(const SweepClass& k, const SweepInst* one, char* ws, const double* theta, int64_t ld_theta,
+                          bool keep, const SweepCtl& ctl, cudaStream_t s);
+cudaError_t sweep_dots(const SweepInst* many, const SweepInst* one, int n, char* ws, cudaStream_t s);
+cudaError_t sweep_reverse(const SweepClass& k, const SweepInst* one, char* ws, const double* theta, int64_t ld_theta,
+                          const SweepCtl& ctl, cudaStream_t s);
+cudaError_t sweep_final(const SweepInst* many, const SweepInst* one, int n, const char* ws, const SweepCtl& ctl,
+                        double* energy, double* grad, int64_t ld_grad, cudaStream_t s);
 
 // Host-side facts the streaming launchers need besides the device descriptor.
 struct StreamPlan {

@@ -907,7 +907,7 @@ cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuf
     k_perm_gather<REAL><<<grid, kStreamThreads, 0, stream>>>(sp.str.perm, d.D, psi, psi_am);
     // with the tensor-core plan (and its workspace) the string-driven kernel sums
     // only the groups outside it
-    const bool tc = REAL && sp.use_tc && b.tc.dig != nullptr;
+    const bool tc = REAL && sp.use_tc && b.has_tc;
     const StrPlan& str = tc ? sp.rest : sp.str;
     if (!tc || sp.has_rest) {
       if (str.Db >= kStrWideDb)
@@ -919,7 +919,8 @@ cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuf
     }
     if constexpr (REAL) {
       if (tc) {
-        const cudaError_t e = tc_hpsi(sp.tc, sp.str, b.tc, d.vals, psi_am, lam_am, sp.has_rest, stream);
+        const TcInst one{sp.tc, b.tc, sp.str.ka, sp.str.kb, d.vals};
+        const cudaError_t e = tc_hpsi(tc_single(sp.tc), &one, b.base, sp.has_rest, stream);
         if (e != cudaSuccess) return e;
       }
     }

@@ -205,10 +205,35 @@ __device__ __forceinline__ uint32_t half2_of(int lo, int hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// ---------------------------------------------------------------- instances
+// A launch serves one instance (many null) or a batch: instance and work item come
+// from the list `work` (tile and row kernels) or from blockIdx.y.
+__device__ __forceinline__ TcScratch scratch_of(const TcInst& I, char* ws) {
+  TcScratch s;
+  s.dig = reinterpret_cast<uint16_t*>(ws + I.off.dig);
+  s.one_a = reinterpret_cast<uint16_t*>(ws + I.off.one_a);
+  s.one_b = reinterpret_cast<uint16_t*>(ws + I.off.one_b);
+  s.pexp = reinterpret_cast<int*>(ws + I.off.pexp);
+  s.aexp = reinterpret_cast<int*>(ws + I.off.aexp);
+  s.ade = reinterpret_cast<int*>(ws + I.off.ade);
+  s.bexp = reinterpret_cast<int*>(ws + I.off.bexp);
+  s.bde = reinterpret_cast<int*>(ws + I.off.bde);
+  s.vi = reinterpret_cast<long long*>(ws + I.off.vi);
+  s.vexp = reinterpret_cast<int*>(ws + I.off.vexp);
+  s.vodd = reinterpret_cast<int*>(ws + I.off.vodd);
+  s.vsum = reinterpret_cast<double*>(ws + I.off.vsum);
+  return s;
+}
+
 // ---------------------------------------------------------------- operand preparation
 // Values of one alpha hop against every beta hop: even and odd parts in fixed
 // point below the item's largest magnitude, that exponent, and sum |even| + |odd|.
-__global__ void __launch_bounds__(256) k_tc_values(const TcPlan tc, const double* __restrict__ vals, TcScratch sc) {
+__global__ void __launch_bounds__(256) k_tc_values(const TcInst* __restrict__ many, const TcInst one, char* ws) {
+  const TcInst& I = many ? many[blockIdx.y] : one;
+  const TcPlan& tc = I.tc;
+  if (int(blockIdx.x) >= tc.items) return;
+  const TcScratch sc = scratch_of(I, ws);
+  const double* vals = I.vals;
   __shared__ double rs[8];
   __shared__ int rm[8];
   const int a = blockIdx.x, R = tc.MT * kRows;
@@ -269,9 +294,13 @@ __device__ __forceinline__ uint32_t sign_mask(uint32_t ka) {
 
 // Digits of one row of psi' (s times psi) below the row's largest magnitude.
 // Bound by its writes: 14 bytes per amplitude for 8 read.
-__global__ void __launch_bounds__(256) k_tc_digits(const TcPlan tc, const uint32_t* __restrict__ ka,
-                                                   const uint32_t* __restrict__ kb, const double* __restrict__ psi_am,
-                                                   TcScratch sc) {
+__global__ void __launch_bounds__(256) k_tc_digits(const TcInst* __restrict__ many, const TcInst one, char* ws) {
+  const TcInst& I = many ? many[blockIdx.y] : one;
+  const TcPlan& tc = I.tc;
+  if (int(blockIdx.x) >= tc.Da) return;
+  const TcScratch sc = scratch_of(I, ws);
+  const uint32_t *ka = I.ka, *kb = I.kb;
+  const double* psi_am = reinterpret_cast<const double*>(ws + I.off.psi_am);
   __shared__ int rm[8];
   const int ja = blockIdx.x, tid = threadIdx.x;
   const double* row = psi_am + int64_t(ja) * tc.Db;
@@ -329,19 +358,16 @@ struct TcShared {          // after the operand buffers and the lambda row
 // against four: 16.1 -> 7.2 ms, together with products issued from straight-line
 // code.
 __global__ void __launch_bounds__(kThreads, 1)
-k_tc_hops(const TcPlan tc, const uint32_t* __restrict__ ka, const uint32_t* __restrict__ kb, const TcScratch sc,
-          double* __restrict__ lam_am, int stages) {
+k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int2* __restrict__ work, int n_work,
+          int stages, int lam_len) {
   extern __shared__ __align__(1024) unsigned char raw[];
   unsigned char* base = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   unsigned char* sA = base;
   unsigned char* sB = sA + kDig * kABytes;
   uint32_t* lam_lo = reinterpret_cast<uint32_t*>(sB + uint32_t(stages) * kBBytes);
-  uint32_t* lam_hi = lam_lo + tc.DbP;
-  TcShared& S = *reinterpret_cast<TcShared*>(lam_hi + tc.DbP);
+  uint32_t* lam_hi = lam_lo + lam_len;
+  TcShared& S = *reinterpret_cast<TcShared*>(lam_hi + lam_len);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int R = tc.MT * kRows;  // entries of dst hold eight strings
-  const int n_tiles = tc.DbP / kTileN;
-
   if (warp == kReadWarps + 4) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&S.tmem))
                  : "memory");
@@ -371,7 +397,15 @@ k_tc_hops(const TcPlan tc, const uint32_t* __restrict__ ka, const uint32_t* __re
   uint32_t ph = 0;         // loaders: parity of the empty wait ^ 1; issuer: parity of the full wait
   uint32_t tph = 0;        // tile parity (issuer and readers)
 
-  for (int ia = blockIdx.x; ia < tc.Da; ia += gridDim.x) {
+  for (int wk = blockIdx.x; wk < n_work; wk += gridDim.x) {
+    const TcInst& I = many ? many[__ldg(&work[wk].x)] : one;
+    const int ia = many ? __ldg(&work[wk].y) : wk;
+    const TcPlan& tc = I.tc;
+    const TcScratch sc = scratch_of(I, ws);
+    const uint32_t *ka = I.ka, *kb = I.kb;
+    double* lam_am = reinterpret_cast<double*>(ws + I.off.lam_am);
+    const int R = tc.MT * kRows;  // entries of dst hold eight strings
+    const int n_tiles = tc.DbP / kTileN;
     // scales of this row: 2^ea above every |V psi'| element, 2^e above every partial sum of lambda'
     if (warp == 0) {
       int top = -100000, bad = 0, odd = 0;
@@ -597,9 +631,17 @@ k_tc_hops(const TcPlan tc, const uint32_t* __restrict__ ka, const uint32_t* __re
 // the sum of its table slots, times 2^fold[col] (the source rows' exponents; null:
 // 1), below the row's largest magnitude 2^oexp; ode: 2^(oexp + ode) bounds the sum
 // of magnitudes. Bound by its writes, 14 bytes per matrix element.
-__global__ void __launch_bounds__(256) k_tc_onespin(const TcOneSpin os, const double* __restrict__ vals,
-                                                    const int* __restrict__ fold, uint16_t* __restrict__ dig, int ld,
-                                                    int* __restrict__ oexp, int* __restrict__ ode) {
+__global__ void __launch_bounds__(256) k_tc_onespin(const TcInst* __restrict__ many, const TcInst one, char* ws,
+                                                    int beta) {
+  const TcInst& I = many ? many[blockIdx.y] : one;
+  const TcOneSpin& os = beta ? I.tc.beta : I.tc.alpha;
+  if (int(blockIdx.x) >= os.n) return;
+  const TcScratch sc = scratch_of(I, ws);
+  const double* vals = I.vals;
+  const int* fold = beta ? nullptr : sc.pexp;
+  uint16_t* dig = beta ? sc.one_b : sc.one_a;
+  int *oexp = beta ? sc.bexp : sc.aexp, *ode = beta ? sc.bde : sc.ade;
+  const int ld = beta ? I.tc.DbP : I.tc.DaP;
   extern __shared__ __align__(16) double srow[];
   __shared__ double rs[8];
   __shared__ int rm[8];
@@ -686,8 +728,8 @@ struct GemmShared {
 };
 
 __global__ void __launch_bounds__(kGemmThreads, 1)
-k_tc_onespin_gemm(const TcPlan tc, const TcScratch sc, const uint32_t* __restrict__ ka,
-                  const uint32_t* __restrict__ kb, double* __restrict__ lam_am, int add) {
+k_tc_onespin_gemm(const TcInst* __restrict__ many, const TcInst one, char* ws, const int2* __restrict__ work,
+                  int n_work, int add) {
   extern __shared__ __align__(1024) unsigned char raw[];
   unsigned char* ring = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   GemmShared& S = *reinterpret_cast<GemmShared*>(ring + kRing * kPairBytes);
@@ -712,11 +754,17 @@ k_tc_onespin_gemm(const TcPlan tc, const TcScratch sc, const uint32_t* __restric
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = S.tmem;
-  const int mts = (tc.Da + kRows - 1) / kRows, nts = tc.DbP / kTileN;
-  const int ch0 = tc.DaP / kChunkK, ch1 = tc.DbP / kChunkK;
   int st = 0;
   uint32_t ph = 0, tph = 0;
-  for (int tile = blockIdx.x; tile < mts * nts; tile += gridDim.x) {
+  for (int wk = blockIdx.x; wk < n_work; wk += gridDim.x) {
+    const TcInst& I = many ? many[__ldg(&work[wk].x)] : one;
+    const int tile = many ? __ldg(&work[wk].y) : wk;
+    const TcPlan& tc = I.tc;
+    const TcScratch sc = scratch_of(I, ws);
+    const uint32_t *ka = I.ka, *kb = I.kb;
+    double* lam_am = reinterpret_cast<double*>(ws + I.off.lam_am);
+    const int mts = (tc.Da + kRows - 1) / kRows;
+    const int ch0 = tc.DaP / kChunkK, ch1 = tc.DbP / kChunkK;
     const int m0 = (tile % mts) * kRows, n0 = (tile / mts) * kTileN;
     if (warp >= 8 && warp < 12) {
       const int pt = tid - 256;
@@ -915,17 +963,20 @@ cudaError_t tc_set_smem_limit(size_t bytes) {
   return e;
 }
 
-cudaError_t tc_hpsi(const TcPlan& tc, const StrPlan& str, const TcScratch& sc, const double* vals,
-                    const double* psi_am, double* lam_am, bool add, cudaStream_t stream) {
-  k_tc_values<<<tc.items, 256, 0, stream>>>(tc, vals, sc);
-  k_tc_digits<<<tc.Da, 256, 0, stream>>>(tc, str.ka, str.kb, psi_am, sc);
-  k_tc_onespin<<<tc.Da, 256, size_t(tc.DaP) * 8, stream>>>(tc.alpha, vals, sc.pexp, sc.one_a, tc.DaP, sc.aexp, sc.ade);
-  k_tc_onespin<<<tc.Db, 256, size_t(tc.DbP) * 8, stream>>>(tc.beta, vals, nullptr, sc.one_b, tc.DbP, sc.bexp, sc.bde);
-  const int tiles = (tc.Da + kRows - 1) / kRows * (tc.DbP / kTileN);
-  k_tc_onespin_gemm<<<tiles < tc.sms ? tiles : tc.sms, kGemmThreads, gemm_smem(), stream>>>(tc, sc, str.ka, str.kb,
-                                                                                          lam_am, add ? 1 : 0);
-  const int grid = tc.Da < tc.sms ? tc.Da : tc.sms;
-  k_tc_hops<<<grid, kThreads, hops_smem(tc.DbP, tc.stages), stream>>>(tc, str.ka, str.kb, sc, lam_am, tc.stages);
+int tc_tiles(const TcPlan& tc) { return (tc.Da + kRows - 1) / kRows * (tc.DbP / kTileN); }
+
+cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, cudaStream_t stream) {
+  const TcInst none{};
+  const TcInst& o = one ? *one : none;
+  const TcInst* many = one ? nullptr : B.insts;
+  const unsigned n = one ? 1u : unsigned(B.n);
+  k_tc_values<<<dim3(unsigned(B.items), n), 256, 0, stream>>>(many, o, ws);
+  k_tc_digits<<<dim3(unsigned(B.Da), n), 256, 0, stream>>>(many, o, ws);
+  k_tc_onespin<<<dim3(unsigned(B.Da), n), 256, size_t(B.DaP) * 8, stream>>>(many, o, ws, 0);
+  k_tc_onespin<<<dim3(unsigned(B.Db), n), 256, size_t(B.DbP) * 8, stream>>>(many, o, ws, 1);
+  const int tg = B.n_tiles < B.sms ? B.n_tiles : B.sms, rg = B.n_rows < B.sms ? B.n_rows : B.sms;
+  k_tc_onespin_gemm<<<tg, kGemmThreads, gemm_smem(), stream>>>(many, o, ws, B.tiles, B.n_tiles, add ? 1 : 0);
+  k_tc_hops<<<rg, kThreads, hops_smem(B.DbP, B.stages), stream>>>(many, o, ws, B.rows, B.n_rows, B.stages, B.DbP);
   return cudaGetLastError();
 }
 
