@@ -5,6 +5,7 @@
 // an unnamed namespace, so each translation unit keeps its own copy.
 #pragma once
 
+#include <climits>
 #include <cuda_runtime.h>
 
 #include "vqe_internal.h"
@@ -55,6 +56,47 @@ __device__ __forceinline__ unsigned long long fix_mag(double x) {
 }
 // 2^e as a double, for |e| < 1000
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double(static_cast<long long>(1023 + e) << 52); }
+// x = h 2^32 + l with both words signed
+struct Words {
+  int h, l;
+};
+__device__ __forceinline__ Words split(long long x) { return {int((x + (1ll << 31)) >> 32), int(uint32_t(x))}; }
+// c a + s b for amplitudes of at most 2^62 (2^62 is 1) and c^2 + s^2 = 1, to one unit:
+// the six products of words that reach the result. Signed low words make the products of
+// two of them, which are left out, as often negative as positive; with unsigned ones (or
+// a low bit dropped) every small amplitude shifts the same way at every gate, and sums
+// over millions of them see that (1e-12 of the energy over 2.7 million states and 144
+// gates).
+__device__ __forceinline__ long long turn(Words a, Words b, int ch, int cl, int sh, int sl) {
+  long long m = static_cast<long long>(a.h) * cl + (1ll << 29);
+  m += static_cast<long long>(b.h) * sl;
+  m += static_cast<long long>(a.l) * ch;
+  m += static_cast<long long>(b.l) * sh;
+  long long p = static_cast<long long>(a.h) * ch;
+  p += static_cast<long long>(b.h) * sh;
+  return (p << 2) + (m >> 30);
+}
+// (a d - b c) / 2^61 in the same way, for |a|, |b| <= 2^62 and |c|, |d| <= 2^61
+__device__ __forceinline__ long long cross_high(Words a, Words d, Words b, Words c) {
+  long long m = static_cast<long long>(a.h) * d.l + (1ll << 28), n = static_cast<long long>(b.h) * c.l;
+  m += static_cast<long long>(a.l) * d.h;
+  n += static_cast<long long>(b.l) * c.h;
+  const long long p = static_cast<long long>(a.h) * d.h - static_cast<long long>(b.h) * c.h;
+  return (p << 3) + ((m - n) >> 29);
+}
+// cos and sin as 62-bit fixed point in two signed words each, x = (h 2^32 + l) 2^-62
+__device__ __forceinline__ int4 fixed_trig(double c, double s) {
+  const long long cf = __double2ll_rn(c * 0x1p62);
+  long long sf = __double2ll_rn(s * 0x1p62);
+  if (int32_t(uint32_t(sf)) == INT_MIN) ++sf;  // both words have a negative
+  return make_int4(int32_t((cf + (1ll << 31)) >> 32), int32_t(uint32_t(cf)), int32_t((sf + (1ll << 31)) >> 32),
+                   int32_t(uint32_t(sf)));
+}
+// e with sqrt(l2) <= 2^e
+__device__ __forceinline__ int norm_exp(double l2) {
+  const int ex = int((__double_as_longlong(l2) >> 52) & 0x7ff);
+  return ex == 0 ? -400 : (ex - 1022 + 1) >> 1;
+}
 // smallest e with b < 2^e for a finite b >= 0 (clamped to [-400, 400])
 __device__ __forceinline__ int bound_exp(double b) {
   const int ex = int((__double_as_longlong(b) >> 52) & 0x7ff);

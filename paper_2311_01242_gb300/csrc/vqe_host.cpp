@@ -1695,7 +1695,7 @@ int run_mid(vqe_hamiltonian_t h, vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e
   if (ce == cudaSuccess) ce = vqe::tc_hpsi(vqe::tc_single(e->tc), &T, ws, false, stream);
   if (ce == cudaSuccess) ce = vqe::sweep_dots(nullptr, &I, 1, ws, stream);
   if (ce == cudaSuccess && grad) ce = vqe::sweep_reverse(k, &I, ws, theta, 0, ctl, stream);
-  if (ce == cudaSuccess) ce = vqe::sweep_final(nullptr, &I, 1, ws, ctl, energy, grad, 0, stream);
+  if (ce == cudaSuccess) ce = vqe::sweep_final(nullptr, &I, 1, ws, theta, 0, ctl, energy, grad, 0, stream);
   return ce == cudaSuccess ? VQE_OK : cuda_fail(ce, "cluster sweeps launch");
 }
 
@@ -3106,7 +3106,8 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
         for (const auto& k : sb.classes)
           if (ce == cudaSuccess) ce = vqe::sweep_reverse(k, nullptr, w, theta, ld_theta, ctl, stream);
       if (ce == cudaSuccess)
-        ce = vqe::sweep_final(sb.d_sweep, nullptr, n, w, ctl, energies, with_grad ? grads : nullptr, ld_grad, stream);
+        ce = vqe::sweep_final(sb.d_sweep, nullptr, n, w, theta, ld_theta, ctl, energies, with_grad ? grads : nullptr,
+                              ld_grad, stream);
       if (ce != cudaSuccess) return cuda_fail(ce, "batched cluster sweeps launch");
     } else {
       for (size_t k = 0; k < sb.mid.size(); ++k) {

@@ -390,8 +390,9 @@ cudaError_t sweep_forward(const SweepClass& k, const SweepInst* one, char* ws, c
 cudaError_t sweep_dots(const SweepInst* many, const SweepInst* one, int n, char* ws, cudaStream_t s);
 cudaError_t sweep_reverse(const SweepClass& k, const SweepInst* one, char* ws, const double* theta, int64_t ld_theta,
                           const SweepCtl& ctl, cudaStream_t s);
-cudaError_t sweep_final(const SweepInst* many, const SweepInst* one, int n, const char* ws, const SweepCtl& ctl,
-                        double* energy, double* grad, int64_t ld_grad, cudaStream_t s);
+cudaError_t sweep_final(const SweepInst* many, const SweepInst* one, int n, const char* ws, const double* theta,
+                        int64_t ld_theta, const SweepCtl& ctl, double* energy, double* grad, int64_t ld_grad,
+                        cudaStream_t s);
 
 // Host-side facts the streaming launchers need besides the device descriptor.
 struct StreamPlan {

@@ -35,33 +35,6 @@ struct GateTab {
   int32_t pad0, pad1;
 };
 
-// c a + s b for amplitudes of at most 2^62 and c^2 + s^2 = 1, to about one unit: the
-// three products of words that reach the result, each pair accumulated by one
-// multiply-add (16 instructions; two full 64 x 64 high products with their sign
-// corrections take over 30). The low words lose a bit so that they stay signed.
-__device__ __forceinline__ long long turn(long long a, long long b, int ch, int cl, int sh, int sl) {
-  const int ah = int(a >> 32), al = int(uint32_t(a) >> 1), bh = int(b >> 32), bl = int(uint32_t(b) >> 1);
-  long long u = static_cast<long long>(al) * ch + (1ll << 28);
-  u += static_cast<long long>(bl) * sh;
-  long long v = static_cast<long long>(ah) * cl;
-  v += static_cast<long long>(bh) * sl;
-  long long p = static_cast<long long>(ah) * ch;
-  p += static_cast<long long>(bh) * sh;
-  return (p << 2) + (((v >> 1) + u) >> 29);
-}
-// (a d - b c) / 2^64 in the same way
-__device__ __forceinline__ long long cross_high(long long a, long long d, long long b, long long c) {
-  const int ah = int(a >> 32), al = int(uint32_t(a) >> 1), dh = int(d >> 32), dl = int(uint32_t(d) >> 1);
-  const int bh = -int(b >> 32), bl = -int(uint32_t(b) >> 1), c_h = int(c >> 32), c_l = int(uint32_t(c) >> 1);
-  long long p = static_cast<long long>(ah) * dh;
-  p += static_cast<long long>(bh) * c_h;
-  long long x = static_cast<long long>(ah) * dl + (1ll << 30);
-  x += static_cast<long long>(al) * dh;
-  x += static_cast<long long>(bh) * c_l;
-  x += static_cast<long long>(bl) * c_h;
-  return p + (x >> 31);
-}
-
 template <int C>
 struct Cluster {
   static __device__ __forceinline__ uint32_t rank() {
@@ -153,13 +126,11 @@ __device__ __forceinline__ void fill_table(GateTab* tab, const int64_t* pair_off
     const int64_t p0 = __ldg(pair_off + m), n = __ldg(pair_off + m + 1) - p0;
     const int64_t lo = n * rank / C, hi = n * (rank + 1) / C;
     GateTab t;
-    const long long cf = __double2ll_rn(c * 0x1p62);
-    long long sf = __double2ll_rn(s * 0x1p62);
-    if (int32_t(uint32_t(sf)) == INT_MIN) ++sf;  // both words have a negative
-    t.ch = int32_t((cf + (1ll << 31)) >> 32);
-    t.cl = int32_t(uint32_t(cf));
-    t.sh = int32_t((sf + (1ll << 31)) >> 32);
-    t.sl = int32_t(uint32_t(sf));
+    const int4 f = fixed_trig(c, s);
+    t.ch = f.x;
+    t.cl = f.y;
+    t.sh = f.z;
+    t.sl = f.w;
     t.lo = int32_t(p0 + lo);
     t.n = int32_t(hi - lo);
     tab[m] = t;
@@ -236,8 +207,9 @@ k_sweep_fwd(const SweepInst* __restrict__ many, const SweepInst one, char* ws, c
     auto rotate = [&](uint32_t px, uint32_t ya, uint32_t yb, long long va, long long vb, int q) {
       const bool neg = int(px) < 0;  // the pair's sign
       const int sh = neg ? -t.sh : t.sh, sl = neg ? -t.sl : t.sl;
-      const long long na = turn(va, vb, t.ch, t.cl, -sh, -sl);
-      const long long nb = turn(vb, va, t.ch, t.cl, sh, sl);
+      const Words wa = split(va), wb = split(vb);
+      const long long na = turn(wa, wb, t.ch, t.cl, -sh, -sl);
+      const long long nb = turn(wb, wa, t.ch, t.cl, sh, sl);
       K::st(ya, na);
       K::st(yb, nb);
       if (keep) __stcg(phi + t.lo + q, make_longlong2(na, nb));
@@ -301,12 +273,6 @@ __device__ __forceinline__ double dot_total(const char* ws, const SweepInst& I, 
   for (int i = 0; i < kDots; ++i) s += p[2 * i];
   return s;
 }
-// e with ||lambda|| <= 2^e
-__device__ __forceinline__ int lambda_exp(double l2) {
-  const int ex = int((__double_as_longlong(l2) >> 52) & 0x7ff);
-  return ex == 0 ? -400 : (ex - 1022 + 1) >> 1;
-}
-
 // Reverse sweep: gradient contributions from the forward sweep's outputs and lambda,
 // then lambda <- U_k^T lambda (inputs copied gates ahead as in the forward sweep).
 template <int C>
@@ -332,7 +298,7 @@ k_sweep_rev(const SweepInst* __restrict__ many, const SweepInst one, char* ws, c
   pdl_release();
   if (ctl.probe >= 0 && rank == 0) probe_wait(ctl, ctl.task0 + ctl.n + I->task);
   fill_table<C>(tab, I->pair_off, M, rank, theta + I->inst * ld_theta);
-  if (tid == 0) scale = pow2(61 - lambda_exp(dot_total(ws, *I, 1)));
+  if (tid == 0) scale = pow2(61 - norm_exp(dot_total(ws, *I, 1)));
   K::sync();  // the other CTAs have started: their shared memory may be written
   const double* lam_am = reinterpret_cast<const double*>(ws + I->lam_am);
   const uint32_t* perm = I->perm;
@@ -397,9 +363,10 @@ k_sweep_rev(const SweepInst* __restrict__ many, const SweepInst one, char* ws, c
     auto step = [&](uint32_t px, longlong2 ph, uint32_t ya, uint32_t yb, long long va, long long vb) {
       const bool neg = int(px) < 0;
       const int sh = neg ? -t.sh : t.sh, sl = neg ? -t.sl : t.sl;
-      K::st(ya, turn(va, vb, t.ch, t.cl, sh, sl));
-      K::st(yb, turn(vb, va, t.ch, t.cl, -sh, -sl));
-      acc += neg_if(cross_high(ph.x, vb, ph.y, va), neg);
+      const Words wa = split(va), wb = split(vb);
+      K::st(ya, turn(wa, wb, t.ch, t.cl, sh, sl));
+      K::st(yb, turn(wb, wa, t.ch, t.cl, -sh, -sl));
+      acc += neg_if(cross_high(split(ph.x), wb, split(ph.y), wa), neg);
     };
 #pragma unroll
     for (int u = 0; u < kAhead; ++u)
@@ -430,19 +397,23 @@ k_sweep_rev(const SweepInst* __restrict__ many, const SweepInst one, char* ws, c
   pdl_wait();
 }
 
-// Energies and gradients; NaN where the batch recorded a failed wait or lambda is
-// not finite.
+// Energies and gradients; NaN where the batch recorded a failed wait, an angle of a
+// gate with pairs is not finite (fixed point holds no NaN) or lambda is not.
 __global__ void __launch_bounds__(256) k_sweep_final(const SweepInst* __restrict__ many, const SweepInst one,
-                                                     const char* ws, const SweepCtl ctl, double* __restrict__ energy,
+                                                     const char* ws, const double* __restrict__ theta, int64_t ld_theta,
+                                                     const SweepCtl ctl, double* __restrict__ energy,
                                                      double* __restrict__ grad, int64_t ld_grad) {
   const SweepInst& I = many ? many[blockIdx.x] : one;
   const double nan = llbits(0x7ff8000000000000ll);
-  const bool lost = ctl.status && *ctl.status != 0;
+  int odd = ctl.status && *ctl.status != 0;
+  for (int m = threadIdx.x; m < I.M; m += 256)
+    odd |= !(fabs(theta[I.inst * ld_theta + m]) < llbits(0x7ff0000000000000ll)) && I.pair_off[m + 1] > I.pair_off[m];
+  const bool lost = __syncthreads_or(odd) != 0;
   if (threadIdx.x == 0) energy[I.inst] = lost ? nan : dot_total(ws, I, 0);
   if (!grad) return;
   const double l2 = dot_total(ws, I, 1);
   const bool bad = lost || !(l2 < llbits(0x7ff0000000000000ll));
-  const double sc = pow2(lambda_exp(l2) - 58);
+  const double sc = pow2(norm_exp(l2) - 61);
   const long long* g = reinterpret_cast<const long long*>(ws + I.gacc);
   for (int m = threadIdx.x; m < I.M; m += 256) grad[I.inst * ld_grad + m] = bad ? nan : __ll2double_rn(g[m]) * sc;
 }
@@ -555,10 +526,11 @@ cudaError_t sweep_reverse(const SweepClass& k, const SweepInst* one, char* ws, c
   }
 }
 
-cudaError_t sweep_final(const SweepInst* many, const SweepInst* one, int n, const char* ws, const SweepCtl& ctl,
-                        double* energy, double* grad, int64_t ld_grad, cudaStream_t s) {
-  k_sweep_final<<<unsigned(n), 256, 0, s>>>(one ? nullptr : many, one ? *one : SweepInst{}, ws, ctl, energy, grad,
-                                            ld_grad);
+cudaError_t sweep_final(const SweepInst* many, const SweepInst* one, int n, const char* ws, const double* theta,
+                        int64_t ld_theta, const SweepCtl& ctl, double* energy, double* grad, int64_t ld_grad,
+                        cudaStream_t s) {
+  k_sweep_final<<<unsigned(n), 256, 0, s>>>(one ? nullptr : many, one ? *one : SweepInst{}, ws, theta, ld_theta, ctl,
+                                            energy, grad, ld_grad);
   return cudaGetLastError();
 }
 
