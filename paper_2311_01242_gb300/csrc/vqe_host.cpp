@@ -357,6 +357,7 @@ struct vqe_ansatz_s {
   uint64_t serial = 0;  // never reused: keys cached batch plans
   std::mutex sweep_mu;
   std::unique_ptr<vqe::SweepPlan> sweep;  // persistent gate sweeps, built on first streaming use
+  std::unique_ptr<vqe::GroupPlan> group;  // gate sweeps by groups, built on first streaming use
   std::tuple<int, int, int> key() const { return std::make_tuple(n, n_elec, n_alpha); }
   ~vqe_ansatz_s() {
     if (sweep) {
@@ -365,6 +366,8 @@ struct vqe_ansatz_s {
       dfree(sweep->d_fwd);
       dfree(sweep->d_adj);
     }
+    if (group)
+      for (void* p : group->alloc) dfree(p);
     dfree(d_gates);
     dfree(d_pair_off);
     dfree(d_chunk_off);
@@ -1114,6 +1117,20 @@ int build_strings(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e
   return VQE_OK;
 }
 
+// Largest instance a persistent slot takes: every per-gate pair list and the
+// sector fit one pass of 1024 blocks of 256 threads, so the slot's reductions
+// follow the single-instance kernels' partial sums exactly.
+constexpr int64_t kSlotMaxItems = int64_t(vqe::kMaxPartials) * vqe::kStreamThreads;
+
+bool slot_fits(vqe_ansatz_t a) {
+  if (int64_t(a->sector.size()) > kSlotMaxItems) return false;
+  for (int m = 0; m < a->M; ++m)
+    if (a->pair_off[m + 1] - a->pair_off[m] > kSlotMaxItems) return false;
+  return true;
+}
+
+size_t binomial(int n, int k);
+
 const vqe_hamiltonian_s::Ell* get_ell(vqe_hamiltonian_t h, vqe_ansatz_t a, int* err) {
   *err = VQE_OK;
   std::lock_guard<std::mutex> lock(h->mu);
@@ -1353,6 +1370,7 @@ struct WsLayout {
   bool has_tc;
   vqe::TcOffsets tc;  // tensor-core H psi
   size_t sw_phi, sw_gacc, sw_dot;  // sweeps in cluster shared memory
+  size_t gr_trig, gr_gacc, gr_norm;  // sweeps by groups of gates
 };
 
 // Real sectors from this size keep the forward sweep's pair outputs for the
@@ -1377,6 +1395,16 @@ bool mid_ansatz(vqe_ansatz_t a) {
          int64_t(a->pairs.size()) < (int64_t(1) << 30);
 }
 
+// Whether the gate sweeps of this ansatz can run in groups (get_groups). A gate of a spin
+// sector touches an eighth of the amplitudes at most, a group of a few gates half of
+// them: from a few million states on, where launches no longer count, a launch per gate
+// moves less.
+constexpr int64_t kGroupSpinStates = int64_t(3) << 19;
+bool group_ansatz(vqe_ansatz_t a) {
+  const int64_t D = int64_t(a->sector.size());
+  return !a->pairs.empty() && D > kSweepStates && (a->n_alpha < 0 || D <= kGroupSpinStates);
+}
+
 WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   WsLayout L;
   const size_t amp = complex_amp ? 16 : 8;
@@ -1390,7 +1418,7 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   L.ctr = L.epart + align256(size_t(vqe::kMaxPartials) * 8);  // task counters of the persistent sweeps
   L.gpart = L.ctr + 256;
   L.phi = L.gpart + (with_grad ? align256(size_t(std::max(a->M, 1)) * vqe::kMaxPartials * 8) : 0);
-  const bool keep = !complex_amp && with_grad && a->sector.size() >= kKeepPhiMinStates;
+  const bool keep = !complex_amp && with_grad && a->sector.size() >= kKeepPhiMinStates && !group_ansatz(a);
   L.total = L.phi + (keep ? align256(size_t(a->pair_off.empty() ? 0 : a->pair_off.back()) * 16) : 0);
   if (!keep) L.phi = 0;
   std::memset(&L.tc, 0, sizeof(L.tc));
@@ -1427,6 +1455,13 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
     L.sw_phi = L.sw_dot + align256(size_t(2 * vqe::kSweepDots) * 8);
     L.total = L.sw_phi + (with_grad ? align256(std::max<size_t>(a->pairs.size(), 1) * 16) : 0);
   }
+  L.gr_trig = L.gr_gacc = L.gr_norm = 0;
+  if (!complex_amp && group_ansatz(a)) {
+    L.gr_norm = L.total;
+    L.gr_trig = L.gr_norm + align256(size_t(vqe::kMaxPartials + 2) * 8);
+    L.gr_gacc = L.gr_trig + align256(size_t(a->M) * 16);
+    L.total = L.gr_gacc + (with_grad ? align256(size_t(a->M) * vqe::kGroupCopies * 8) : 0);
+  }
   return L;
 }
 
@@ -1441,6 +1476,12 @@ vqe::StreamBuffers buffers(void* ws, const WsLayout& L) {
   s.epart = reinterpret_cast<double*>(b + L.epart);
   s.gpart = reinterpret_cast<double*>(b + L.gpart);
   s.phi = L.phi ? reinterpret_cast<double2*>(b + L.phi) : nullptr;
+  if (L.gr_trig) {
+    s.group.trig = reinterpret_cast<int4*>(b + L.gr_trig);
+    s.group.gacc = reinterpret_cast<unsigned long long*>(b + L.gr_gacc);
+    s.group.norm = reinterpret_cast<double*>(b + L.gr_norm);
+    s.group.bad = reinterpret_cast<int*>(s.group.norm + vqe::kMaxPartials + 1);
+  }
   s.base = b;
   s.has_tc = L.has_tc;
   s.tc = L.tc;
@@ -1518,8 +1559,205 @@ const vqe::SweepPlan* get_sweep(vqe_ansatz_t a) {
   return ok ? a->sweep.get() : nullptr;
 }
 
-vqe::StreamPlan plan(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e) {
+// Tables of the gate sweeps by groups: consecutive gates while the blocks that their
+// qubits leave stay within kGroupStates amplitudes (fewer groups are fewer passes over
+// the state); then the lowest other qubits, whose amplitudes are neighbours, up to the
+// same bound. Built once per ansatz, on its first use outside a stream capture; null
+// before that, or if the device refuses (the caller then launches per gate).
+struct GroupBuild {
+  uint32_t set = 0;
+  std::vector<int> gates;
+  std::vector<vqe::GroupClass> classes;  // offsets within this group's arrays
+  std::vector<vqe::GroupWork> work;
+  std::vector<int2> ranges;
+  std::vector<uint32_t> patterns, states, pairs;
+  int most = 0, most_pairs = 0;
+};
+// The most ways, over the electron counts r that s of n qubits can hold of k, to place
+// r - f / 2 electrons on s - f qubits: local states (f = 0), or pairs of a gate that
+// flips f qubits.
+size_t most_ways(int s, int k, int n, int f) {
+  size_t b = 0;
+  for (int r = std::max(0, k - (n - s)); r <= std::min(s, k); ++r) b = std::max(b, binomial(s - f, r - f / 2));
+  return b;
+}
+bool group_fits(vqe_ansatz_t a, uint32_t set, const std::vector<int>& gates) {
+  const uint32_t even = uint32_t((uint64_t(1) << a->n) - 1) & 0x55555555u;
+  const int na = pc32(even), nb = a->n - na, sa = pc32(set & even), sb = pc32(set & ~even);
+  auto ways = [&](uint32_t flip) {
+    if (a->n_alpha < 0) return most_ways(sa + sb, a->n_elec, a->n, pc32(flip));
+    return most_ways(sa, a->n_alpha, na, pc32(flip & even)) *
+           most_ways(sb, a->n_elec - a->n_alpha, nb, pc32(flip & ~even));
+  };
+  size_t pairs = 0;
+  for (int m : gates) pairs += ways(a->gates[size_t(m)].flip);
+  return pairs <= size_t(vqe::kGroupPairs) && std::min(ways(0), 2 * pairs) <= size_t(vqe::kGroupStates) &&
+         ways(0) < size_t(1) << 15;
+}
+void build_group(vqe_ansatz_t a, GroupBuild* b) {
+  const uint32_t all = uint32_t((uint64_t(1) << a->n) - 1), even = all & 0x55555555u, set = b->set, env = all & ~set;
+  const bool spin = a->n_alpha >= 0;
+  // electrons a pattern holds: (alpha, beta) in a spin sector, else (all, 0); a difference
+  // with a negative part has no local states (parts are at most 32)
+  auto count = [&](uint32_t k) { return spin ? pc32(k & even) * 64 + pc32(k & ~even) : pc32(k) * 64; };
+  const int full = spin ? a->n_alpha * 64 + (a->n_elec - a->n_alpha) : a->n_elec * 64;
+  auto local_bits = [&](uint32_t k) {  // k's bits on the set, packed
+    uint32_t r = 0, j = 0;
+    for (uint32_t m = set; m; m &= m - 1, ++j) r |= ((k >> __builtin_ctz(m)) & 1u) << j;
+    return r;
+  };
+  // local states by count; at[p]: number of packed pattern p among those of its count
+  std::map<int, std::vector<uint32_t>> packed;
+  std::map<int, std::vector<uint32_t>> patterns;  // of the other qubits, by the count they leave
+  std::vector<uint32_t> dep(size_t(1) << pc32(set)), at(dep.size());
+  uint32_t k = 0;
+  for (size_t p = 0; p < dep.size(); ++p, k = (k - set) & set) {
+    dep[p] = k;
+    auto& v = packed[count(k)];
+    at[p] = uint32_t(v.size());
+    v.push_back(uint32_t(p));
+  }
+  k = 0;
+  for (uint64_t i = 0; i < (uint64_t(1) << pc32(env)); ++i, k = (k - env) & env) {
+    const auto it = packed.find(full - count(k));
+    if (it == packed.end()) continue;
+    patterns[it->first].push_back(k);
+  }
+  // a CTA's share: up to the bound where blocks are small, but enough CTAs to fill the chip
+  const size_t share = std::min(size_t(vqe::kGroupStates), a->sector.size() / vqe::kGroupCtas + 1);
+  for (const auto& pt : patterns) {
+    const std::vector<uint32_t>& of = packed[pt.first];
+    vqe::GroupClass c{0, int32_t(b->states.size()), int32_t(b->ranges.size()), int32_t(b->pairs.size()), 0, 0};
+    std::vector<uint32_t> list;
+    std::vector<int32_t> place(of.size(), -1);  // among the states that a gate rotates
+    for (int m : b->gates) {
+      const GateRec& g = a->gates[size_t(m)];
+      const uint32_t occ = a->pairs[size_t(a->pair_off[size_t(m)])] & g.flip;
+      const uint32_t f = local_bits(g.flip), o = local_bits(occ);
+      const int32_t first = int32_t(list.size());
+      for (uint32_t p : of)
+        if ((p & f) == o) {
+          const uint32_t s = uint32_t((pc32(dep[p] & g.par) & 1) ^ (g.sign0 < 0 ? 1 : 0));
+          list.push_back(at[p] | (at[p ^ f] << 15) | (s << 30));
+          place[at[p]] = place[at[p ^ f]] = 0;
+        }
+      b->ranges.push_back(make_int2(first, int32_t(list.size()) - first));
+    }
+    if (list.empty()) {
+      b->ranges.resize(size_t(c.range0));
+      continue;
+    }
+    for (size_t i = 0; i < of.size(); ++i)
+      if (place[i] == 0) {
+        place[i] = c.n++;
+        b->states.push_back(dep[of[i]]);
+      }
+    const int32_t n = c.n;
+    c.inv = 0xffffffffu / uint32_t(n) + 1u;
+    for (uint32_t v : list) {
+      const uint32_t x = uint32_t(place[v & 0x7fffu]), y = uint32_t(place[(v >> 15) & 0x7fffu]);
+      b->pairs.push_back((v >> 30) ? y | x << 16 : x | y << 16);
+    }
+    while (b->pairs.size() % 4) b->pairs.push_back(0);
+    c.pairs = int32_t(b->pairs.size()) - c.pair0;
+    b->most_pairs = std::max(b->most_pairs, c.pairs);
+    const int32_t each = int32_t(std::max<size_t>(1, std::min(size_t(vqe::kGroupPatterns), share / size_t(n))));
+    const int32_t first = int32_t(b->patterns.size()), all_of = int32_t(pt.second.size());
+    for (int32_t i = 0; i < all_of; i += each)
+      b->work.push_back(vqe::GroupWork{int32_t(b->classes.size()), first + i, std::min(each, all_of - i), 0});
+    b->patterns.insert(b->patterns.end(), pt.second.begin(), pt.second.end());
+    b->classes.push_back(c);
+  }
+  auto size = [&](const vqe::GroupWork& w) { return w.count * b->classes[size_t(w.cls)].n; };
+  std::stable_sort(b->work.begin(), b->work.end(),
+                   [&](const vqe::GroupWork& x, const vqe::GroupWork& y) { return size(x) > size(y); });
+  b->most = b->work.empty() ? 0 : (size(b->work[0]) + 3) / 4 * 4;
+}
+const vqe::GroupPlan* get_groups(vqe_ansatz_t a, cudaStream_t stream) {
+  std::lock_guard<std::mutex> lk(a->sweep_mu);
+  if (a->group) return a->group->steps.empty() ? nullptr : a->group.get();
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  std::vector<GroupBuild> b;
+  for (int m = 0; m < a->M; ++m) {
+    if (a->pair_off[size_t(m) + 1] == a->pair_off[size_t(m)]) continue;
+    const uint32_t flip = a->gates[size_t(m)].flip;
+    bool joins = !b.empty() && int(b.back().gates.size()) < vqe::kGroupGates;
+    if (joins) {
+      b.back().gates.push_back(m);
+      joins = group_fits(a, b.back().set | flip, b.back().gates);
+      if (!joins) b.back().gates.pop_back();
+    }
+    if (!joins) {
+      b.emplace_back();
+      b.back().gates.push_back(m);
+    }
+    b.back().set |= flip;
+  }
+  for (GroupBuild& g : b)
+    for (int q = 0; q < a->n; ++q)
+      if (group_fits(a, g.set | (1u << q), g.gates)) g.set |= 1u << q;
+  parallel_items(int64_t(b.size()), [&](int64_t i) { build_group(a, &b[size_t(i)]); });
+  std::unique_ptr<vqe::GroupPlan> p(new vqe::GroupPlan);
+  std::vector<vqe::GroupGate> gates;
+  std::vector<vqe::GroupClass> classes;
+  std::vector<vqe::GroupWork> work;
+  std::vector<int2> ranges;
+  std::vector<uint32_t> patterns, states, pairs;
+  for (const GroupBuild& g : b) {
+    const int32_t c0 = int32_t(classes.size()), s0 = int32_t(states.size()), r0 = int32_t(ranges.size()),
+                  p0 = int32_t(pairs.size()), t0 = int32_t(patterns.size());
+    p->steps.push_back(vqe::GroupStep{int32_t(gates.size()), int32_t(g.gates.size()), int32_t(work.size()),
+                                      int32_t(g.work.size()), g.most, g.most_pairs});
+    for (int m : g.gates) gates.push_back(vqe::GroupGate{m, a->gates[size_t(m)].par & ~g.set});
+    for (vqe::GroupClass c : g.classes) {
+      c.state0 += s0;
+      c.range0 += r0;
+      c.pair0 += p0;
+      classes.push_back(c);
+    }
+    for (vqe::GroupWork x : g.work) {
+      x.cls += c0;
+      x.first += t0;
+      work.push_back(x);
+    }
+    patterns.insert(patterns.end(), g.patterns.begin(), g.patterns.end());
+    ranges.insert(ranges.end(), g.ranges.begin(), g.ranges.end());
+    states.insert(states.end(), g.states.begin(), g.states.end());
+    pairs.insert(pairs.end(), g.pairs.begin(), g.pairs.end());
+  }
+  vqe::GroupTables& t = p->tables;
+  auto put = [&](const auto& v, auto** dst) {
+    typename std::remove_const<typename std::remove_pointer<decltype(v.data())>::type>::type* d = nullptr;
+    if (upload(v, &d) != VQE_OK) return false;
+    p->alloc.push_back(d);
+    *dst = d;
+    return true;
+  };
+  const bool ok = pairs.size() < size_t(INT32_MAX) && states.size() < size_t(INT32_MAX) &&
+                  vqe::group_set_limits() == cudaSuccess && put(gates, &t.gates) && put(classes, &t.classes) &&
+                  put(work, &t.work) && put(patterns, &t.patterns) && put(ranges, &t.ranges) && put(states, &t.states) && put(pairs, &t.pairs);
+  t.rank_hi = a->d_rank_hi;
+  t.rank_lo = a->d_rank_lo;
+  t.lo_bits = a->lo_bits;
+  if (!ok) {
+    cudaGetLastError();
+    for (void* d : p->alloc) dfree(d);
+    p.reset(new vqe::GroupPlan);
+  }
+  a->group = std::move(p);
+  return ok ? a->group.get() : nullptr;
+}
+
+// Launches of one streamed evaluation. FP64 sweeps, complex amplitudes and small
+// sectors run one launch per gate.
+vqe::StreamPlan plan(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, cudaStream_t stream, bool sweeps = true) {
   vqe::StreamPlan p;
+  if (sweeps && use_real() && !(g_flags & VQE_FLAG_FP64_SWEEPS) && group_ansatz(a) && (e->use_tc || !slot_fits(a)))
+    p.group = get_groups(a, stream);  // (a batch's slots sweep in FP64, with the same bits as single calls)
   if (use_real() && (g_flags & VQE_FLAG_PERSISTENT_SWEEPS)) {
     p.sweep = get_sweep(a);
     p.counters_off = int64_t(ws_layout(a, false, false).ctr);
@@ -1721,7 +1959,7 @@ int run_single(vqe_hamiltonian_t h, vqe_ansatz_t a, const double* theta, double*
   if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
   if (mid_flags() && mid_fits(a, e))
     return run_mid(h, a, e, d, theta, energy, with_grad ? grad : nullptr, static_cast<char*>(ws), L, stream);
-  cudaError_t ce = stream_eval(d, plan(a, e), buffers(ws, L), real, with_grad, theta, energy, grad, stream);
+  cudaError_t ce = stream_eval(d, plan(a, e, stream), buffers(ws, L), real, with_grad, theta, energy, grad, stream);
   if (ce != cudaSuccess) return cuda_fail(ce, "streaming launch");
   return VQE_OK;
 }
@@ -1749,7 +1987,7 @@ int prepare_noalloc(vqe_hamiltonian_s* h, vqe_ansatz_s* a, bool with_grad, size_
     if (it != h->ells.end()) e = &it->second;  // entries are never erased while h lives
   }
   *d = make_desc(h, a, e, 0);
-  *sp = plan(a, e);
+  *sp = plan(a, e, nullptr, false);
   sp->use_tc = false;  // its operands do not fit the scratch
   sp->sweep = nullptr;  // one launch per gate: the sweep queues address the regular workspace layout
   // the string-driven H psi needs two more sector-sized vectors; when they do
@@ -2463,6 +2701,7 @@ size_t vqe_workspace_bytes(vqe_hamiltonian_t h, vqe_ansatz_t a, int mode) {
   if (!get_ell(h, a, &rc)) return 0;
   const bool cplx_amp = (mode & VQE_WS_COMPLEX) || !use_real();
   if (!cplx_amp && (g_flags & VQE_FLAG_PERSISTENT_SWEEPS)) get_sweep(a);  // before any stream capture
+  if (!cplx_amp && group_ansatz(a)) get_groups(a, nullptr);
   return ws_layout(a, cplx_amp, (mode & VQE_WS_GRAD) != 0).total;
 }
 
@@ -2486,7 +2725,7 @@ int vqe_state(vqe_ansatz_t a, vqe_hamiltonian_t h, const double* theta, double* 
   const WsLayout L = ws_layout(a, false, false);
   if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
   InstDesc d = make_desc(h, a, e, 0);
-  cudaError_t ce = vqe::stream_state(d, plan(a, e), buffers(ws, L), theta, psi_out,
+  cudaError_t ce = vqe::stream_state(d, plan(a, e, static_cast<cudaStream_t>(stream)), buffers(ws, L), theta, psi_out,
                                      static_cast<cudaStream_t>(stream));
   if (ce != cudaSuccess) return cuda_fail(ce, "state launch");
   return VQE_OK;
@@ -2502,7 +2741,7 @@ int vqe_apply_hamiltonian(vqe_hamiltonian_t h, vqe_ansatz_t a, const double* psi
   const WsLayout L = ws_layout(a, true, false);
   if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
   InstDesc d = make_desc(h, a, e, 0);
-  cudaError_t ce = vqe::stream_apply_h(d, plan(a, e), buffers(ws, L), psi, lam_out, energy,
+  cudaError_t ce = vqe::stream_apply_h(d, plan(a, e, nullptr, false), buffers(ws, L), psi, lam_out, energy,
                                        static_cast<cudaStream_t>(stream));
   if (ce != cudaSuccess) return cuda_fail(ce, "apply_hamiltonian launch");
   return VQE_OK;
@@ -2522,7 +2761,7 @@ int vqe_apply_hamiltonian_sector(vqe_hamiltonian_t h, vqe_ansatz_t a, const doub
   vqe::StreamBuffers b = buffers(ws, L);
   b.psi = const_cast<double*>(psi);  // read only: H psi writes lambda and the alpha-major copies
   b.lam = lam_out;
-  cudaError_t ce = vqe::stream_apply_h_real(d, plan(a, e), b, energy, static_cast<cudaStream_t>(stream));
+  cudaError_t ce = vqe::stream_apply_h_real(d, plan(a, e, nullptr, false), b, energy, static_cast<cudaStream_t>(stream));
   if (ce != cudaSuccess) return cuda_fail(ce, "apply_hamiltonian_sector launch");
   return VQE_OK;
 }
@@ -2561,7 +2800,7 @@ int vqe_pool_gradients(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_ansatz_t pool, c
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   InstDesc d = make_desc(h, a, e, 0);
   const vqe::StreamBuffers b = buffers(ws, L);
-  cudaError_t ce = vqe::stream_energy_grad(d, plan(a, e), b, real, false, theta, energy, nullptr, st);
+  cudaError_t ce = vqe::stream_energy_grad(d, plan(a, e, st), b, real, false, theta, energy, nullptr, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "pool screening forward / H psi launch");
   double* part = reinterpret_cast<double*>(static_cast<char*>(ws) + L.total);
   void* pl = static_cast<char*>(ws) + L.total + part_bytes;
@@ -2569,18 +2808,6 @@ int vqe_pool_gradients(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_ansatz_t pool, c
                            b.lam, int64_t(a->sector.size()), pl, part, pool_grad, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "pool screening launch");
   return VQE_OK;
-}
-
-// Largest instance a persistent slot takes: every per-gate pair list and the
-// sector fit one pass of 1024 blocks of 256 threads, so the slot's reductions
-// follow the single-instance kernels' partial sums exactly.
-constexpr int64_t kSlotMaxItems = int64_t(vqe::kMaxPartials) * vqe::kStreamThreads;
-
-static bool slot_fits(vqe_ansatz_t a) {
-  if (int64_t(a->sector.size()) > kSlotMaxItems) return false;
-  for (int m = 0; m < a->M; ++m)
-    if (a->pair_off[m + 1] - a->pair_off[m] > kSlotMaxItems) return false;
-  return true;
 }
 
 // Builds both task queues of the persistent launch for the current grid and
@@ -2922,6 +3149,8 @@ static int build_stream_batch(vqe_batch_s* B) {
     else
       sb.big.push_back(i);
   }
+  for (int i : sb.big)
+    if (group_ansatz(B->ans[i])) get_groups(B->ans[i], nullptr);
   for (int i : sb.big) sb.big_bytes = std::max(sb.big_bytes, ws_layout(B->ans[i], false, true).total);
   const int n = int(sb.slots.size());
   if (n == 0 && sb.mid.empty()) return VQE_OK;
@@ -3038,7 +3267,7 @@ static int run_one_by_one(vqe_batch_t b, const std::vector<int>& which, bool rea
     if (!e) return rc2;
     const WsLayout L = ws_layout(a, !real, with_grad);
     if ((rc2 = check_ws(ws, ws_bytes, L.total))) return rc2;
-    cudaError_t ce = stream_eval(b->descs[i], plan(a, e), buffers(ws, L), real, with_grad,
+    cudaError_t ce = stream_eval(b->descs[i], plan(a, e, stream), buffers(ws, L), real, with_grad,
                                  theta + int64_t(i) * ld_theta, energies + i,
                                  with_grad ? grads + int64_t(i) * ld_grad : nullptr, stream);
     if (ce != cudaSuccess) return cuda_fail(ce, "batched streaming launch");

@@ -5,6 +5,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <vector>
 
 struct vqe_hamiltonian_s;
 struct vqe_ansatz_s;
@@ -342,6 +343,61 @@ cudaError_t launch_resident(const InstDesc* d_descs, const InstDesc* one, int n_
                             cudaStream_t stream, int ctas_per_instance, bool fixed_point);
 cudaError_t set_resident_smem_limit(size_t smem, bool real);
 
+// Gate sweeps of large real instances in groups of gates (vqe_group.cu).
+constexpr int kGroupThreads = 512;
+constexpr int kGroupStates = 3456;   // amplitudes per CTA: three or four CTAs per SM with psi and lambda
+constexpr int kGroupPatterns = 256;  // blocks per CTA
+constexpr int kGroupPairs = 8192;    // pair-list entries of a class (all gates of the group)
+constexpr int kGroupGates = 32;      // gates per group
+constexpr int kGroupCtas = 304;      // two per SM: the next group's can start beside them
+constexpr int kGroupCopies = 32;     // of the gradient sums, so that blocks rarely meet at one
+struct GroupGate {
+  int32_t m;         // angle
+  uint32_t par;      // qubits outside the group's set in the gate's sign
+};
+struct GroupClass {  // blocks with the same electron counts on the group's qubits
+  int32_t n, state0, range0;  // local states states[state0 ...]; ranges[range0 + gate of the group]
+  int32_t pair0, pairs;       // pairs[pair0 ...], a multiple of four, padded to one
+  uint32_t inv;               // 2^32 / n, rounded up
+};
+struct GroupWork {            // a CTA's blocks: patterns[first, first + count) of one class
+  int32_t cls, first, count, pad;
+};
+struct GroupTables {
+  const GroupGate* gates;
+  const GroupClass* classes;
+  const GroupWork* work;     // the largest first
+  const uint32_t* patterns;  // occupations of the other qubits
+  const int2* ranges;        // first pair (within the class's) and number of pairs
+  const uint32_t* states;    // occupation of the group's qubits, increasing
+  const uint32_t* pairs;     // local state | state after the flip << 16, swapped where the local sign is -1
+  const uint32_t* rank_hi;
+  const uint32_t* rank_lo;
+  int32_t lo_bits;
+};
+struct GroupStep {           // one group
+  int32_t gate0, gates, work0, ctas;
+  int32_t most, most_pairs;  // amplitudes of the largest CTA, a multiple of four; padded pairs of a class
+};
+struct GroupPlan {
+  GroupTables tables{};
+  std::vector<GroupStep> steps;
+  std::vector<void*> alloc;  // device arrays behind tables
+};
+struct GroupBuffers {
+  int4* trig;                // [M]
+  unsigned long long* gacc;  // [kGroupCopies][M]
+  double* norm;              // <lambda|lambda>, then kMaxPartials partial sums of it
+  int* bad;
+};
+cudaError_t group_set_limits();
+// psi (FP64, sector order) after the gates; with_grad: also clears the gradient sums
+cudaError_t group_forward(const InstDesc& d, const GroupPlan& p, const GroupBuffers& w, const double* theta,
+                          double* psi, bool with_grad, cudaStream_t stream);
+// the gradient from that psi and lambda; scratch: 2 D doubles, 16-byte aligned
+cudaError_t group_reverse(const InstDesc& d, const GroupPlan& p, const GroupBuffers& w, const double* psi,
+                          const double* lam, void* scratch, double* grad, cudaStream_t stream);
+
 struct StreamBuffers {
   void* psi = nullptr;     // D amplitudes (double or double2), sector order
   void* lam = nullptr;     // D amplitudes
@@ -350,6 +406,7 @@ struct StreamBuffers {
   // large real instances: the forward sweep's outputs {phi(k), phi(k ^ flip)} of
   // every pair, in pair order (null: the reverse sweep un-applies the gates to psi)
   double2* phi = nullptr;
+  GroupBuffers group{};    // with StreamPlan::group
   char* base = nullptr;    // the workspace
   bool has_tc = false;     // ... has the tensor-core H psi's part, at
   TcOffsets tc{};
@@ -397,6 +454,7 @@ cudaError_t sweep_final(const SweepInst* many, const SweepInst* one, int n, cons
 // Host-side facts the streaming launchers need besides the device descriptor.
 struct StreamPlan {
   const SweepPlan* sweep = nullptr;  // persistent gate sweeps (null: one launch per gate)
+  const GroupPlan* group = nullptr;  // gate sweeps by groups (real amplitudes; before sweep)
   int64_t counters_off = 0;          // byte offset of the sweep queue's counters in the workspace
   const int64_t* pair_off_host;  // [M+1]
   const int32_t* d_nb_rows;      // device [M+1]: blocks of each gate's adjoint launch, then of H psi

@@ -872,8 +872,10 @@ cudaError_t sweep_launch(const StreamPlan& sp, const StreamBuffers& b, bool adjo
 
 template <bool REAL>
 cudaError_t stream_forward(const InstDesc& d, const StreamPlan& sp, const StreamBuffers& b,
-                           const double* theta, cudaStream_t stream) {
+                           const double* theta, bool with_grad, cudaStream_t stream) {
   typedef typename Amp<REAL>::T T;
+  if (REAL && sp.group)
+    return group_forward(d, *sp.group, b.group, theta, static_cast<double*>(b.psi), with_grad, stream);
   if (REAL && sp.sweep) return sweep_launch(sp, b, false, theta, stream);
   T* psi = static_cast<T*>(b.psi);
   const int nt = kStreamThreads;
@@ -941,6 +943,9 @@ cudaError_t stream_adjoint(const InstDesc& d, const StreamPlan& sp, const Stream
   typedef typename Amp<REAL>::T T;
   T* phi = static_cast<T*>(b.psi);
   T* lam = static_cast<T*>(b.lam);
+  if (REAL && sp.group)
+    return group_reverse(d, *sp.group, b.group, static_cast<const double*>(b.psi), static_cast<const double*>(b.lam),
+                         b.psi_am, grad, stream);  // psi_am and lam_am are free again, and neighbours
   if (REAL && sp.sweep) {
     const cudaError_t e = sweep_launch(sp, b, true, nullptr, stream);
     if (e != cudaSuccess) return e;
@@ -964,11 +969,11 @@ cudaError_t stream_energy_grad(const InstDesc& d, const StreamPlan& sp, const St
                                double* grad, cudaStream_t stream) {
   cudaError_t e;
   if (real) {
-    if ((e = stream_forward<true>(d, sp, b, theta, stream)) != cudaSuccess) return e;
+    if ((e = stream_forward<true>(d, sp, b, theta, with_grad, stream)) != cudaSuccess) return e;
     if ((e = stream_hpsi<true>(d, sp, b, energy, stream)) != cudaSuccess) return e;
     if (with_grad) return stream_adjoint<true>(d, sp, b, grad, stream);
   } else {
-    if ((e = stream_forward<false>(d, sp, b, theta, stream)) != cudaSuccess) return e;
+    if ((e = stream_forward<false>(d, sp, b, theta, with_grad, stream)) != cudaSuccess) return e;
     if ((e = stream_hpsi<false>(d, sp, b, energy, stream)) != cudaSuccess) return e;
     if (with_grad) return stream_adjoint<false>(d, sp, b, grad, stream);
   }
@@ -977,7 +982,7 @@ cudaError_t stream_energy_grad(const InstDesc& d, const StreamPlan& sp, const St
 
 cudaError_t stream_state(const InstDesc& d, const StreamPlan& sp, const StreamBuffers& b,
                          const double* theta, double* psi_out, cudaStream_t stream) {
-  cudaError_t e = stream_forward<true>(d, sp, b, theta, stream);
+  cudaError_t e = stream_forward<true>(d, sp, b, theta, false, stream);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(psi_out, 0, (size_t(1) << d.n) * sizeof(double2), stream);
   if (e != cudaSuccess) return e;
