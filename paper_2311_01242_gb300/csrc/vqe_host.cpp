@@ -307,6 +307,9 @@ struct vqe_hamiltonian_s {
     bool use_tc = false, has_rest = false;
     vqe::TcPlan tc{};
     vqe::StrPlan rest{};
+    // large electron-number sectors of counting and hopping Hamiltonians
+    bool use_hop = false;
+    vqe::HopPlan hop;
   };
   std::mutex mu;
   std::map<std::tuple<int, int, int>, Ell> ells;
@@ -1131,6 +1134,161 @@ bool slot_fits(vqe_ansatz_t a) {
 
 size_t binomial(int n, int k);
 
+// Passes of the H psi by hops (HopPlan) of an electron-number sector; none if a group
+// is neither the diagonal nor a plain hop. Sets of qubits grow by the qubit that brings
+// the most hops not yet taken, while blocks stay within kHopStates amplitudes.
+int build_hops(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e) {
+  const int n = a->n, ne = a->n_elec, G = int(h->groups.size());
+  const size_t D = a->sector.size();
+  vqe::HopPlan plan;
+  plan.diag.slot = -1;
+  std::vector<int> left;
+  for (int i = 0; i < G; ++i) {
+    const GroupRec& g = h->groups[size_t(i)];
+    const uint32_t em = h->emask[size_t(g.ebeg)];
+    if (g.x == 0 && g.kind == 2 && em == 0 && plan.diag.slot < 0)
+      plan.diag = vqe::HopDiag{g.vbeg, g.nq, h->emask[size_t(g.ebeg) + 1]};
+    else if (pc32(g.x) == 2 && g.kind == 0 && g.eend == g.ebeg + 1 && g.ubits == 2 && em == 0)
+      left.push_back(i);
+    else
+      return VQE_OK;
+  }
+  // the diagonal's tables go into the workspace's alpha-major vectors
+  if (left.empty() || (size_t(2 + n - a->lo_bits) << a->lo_bits) > 2 * D) return VQE_OK;
+  auto largest = [&](uint32_t set) {
+    size_t b = 0;
+    for (int r = std::max(0, ne - (n - pc32(set))); r <= std::min(pc32(set), ne); ++r)
+      b = std::max(b, binomial(pc32(set), r));
+    return b;
+  };
+  // one CTA per SM at least, before fewer passes
+  const size_t bound = std::min(size_t(vqe::kHopStates), std::max<size_t>(D / 152, 1024));
+  const uint32_t all = uint32_t((uint64_t(1) << n) - 1);
+  std::vector<vqe::HopClass> classes;
+  std::vector<vqe::GroupWork> work;
+  std::vector<uint32_t> patterns, states, list;
+  std::vector<int32_t> slots;
+  while (!left.empty()) {
+    uint32_t set = 0;
+    for (;;) {
+      int best = -1, most = -1;
+      for (int q = 0; q < n; ++q) {
+        const uint32_t s = set | (1u << q);
+        if (s == set || largest(s) > bound) continue;
+        int gain = 0, near = 0;  // hops it completes; failing that, hops that touch it
+        for (int i : left) {
+          const uint32_t x = h->groups[size_t(i)].x;
+          gain += (x & ~s) == 0 && (x & ~set) != 0;
+          near += ((x >> q) & 1u) != 0;
+        }
+        if (gain * 1024 + near > most) {
+          most = gain * 1024 + near;
+          best = q;
+        }
+      }
+      if (best < 0) break;
+      set |= 1u << best;
+    }
+    std::vector<int> hops, rest;
+    for (int i : left)
+      ((h->groups[size_t(i)].x & ~set) == 0 && int(hops.size()) < vqe::kHopSlots / 2 ? hops : rest).push_back(i);
+    if (hops.empty()) return VQE_OK;
+    left.swap(rest);
+    vqe::HopStep step{int32_t(work.size()), 0, 0, int32_t(slots.size()), int32_t(2 * hops.size())};
+    for (int i : hops) {
+      const GroupRec& g = h->groups[size_t(i)];
+      const uint32_t lower = g.x & (0u - g.x);
+      slots.push_back(g.vbeg + int32_t(pattern_bits(g, lower)));
+      slots.push_back(g.vbeg + int32_t(pattern_bits(g, g.x ^ lower)));
+    }
+    const uint32_t env = all & ~set;
+    const int ns = pc32(set);
+    auto packed = [&](uint32_t k) {
+      uint32_t r = 0, j = 0;
+      for (uint32_t m = set; m; m &= m - 1, ++j) r |= ((k >> __builtin_ctz(m)) & 1u) << j;
+      return r;
+    };
+    std::vector<uint32_t> flip, low;
+    for (int i : hops) {
+      const uint32_t x = h->groups[size_t(i)].x;
+      flip.push_back(packed(x));
+      low.push_back(packed(x & (0u - x)));
+    }
+    std::vector<std::vector<uint32_t>> of(size_t(ns) + 1), dep(size_t(ns) + 1), pats(size_t(ns) + 1);
+    std::vector<uint32_t> at(size_t(1) << ns);
+    uint32_t k = 0;
+    for (uint32_t p = 0; p < (1u << ns); ++p, k = (k - set) & set) {
+      const int r = pc32(p);
+      at[p] = uint32_t(of[size_t(r)].size());
+      of[size_t(r)].push_back(p);
+      dep[size_t(r)].push_back(k);
+    }
+    k = 0;
+    for (uint64_t i = 0; i < (uint64_t(1) << pc32(env)); ++i, k = (k - env) & env) {
+      const int r = ne - pc32(k);
+      if (r >= 0 && r <= ns) pats[size_t(r)].push_back(k);
+    }
+    const size_t share = std::min(size_t(vqe::kHopStates), D / vqe::kGroupCtas + 1);
+    for (int r = 0; r <= ns; ++r) {
+      const auto& o = of[size_t(r)];
+      if (pats[size_t(r)].empty()) continue;
+      int width = 0;
+      for (uint32_t p : o) {
+        int w = 0;
+        for (uint32_t x : flip) w += pc32(p & x) == 1;
+        width = std::max(width, w);
+      }
+      if (width == 0) continue;
+      width = vqe::hop_width(width);
+      const int32_t m = int32_t(o.size());
+      const vqe::HopClass c{m, int32_t(states.size()), width, m > 1 ? 0xffffffffu / uint32_t(m) + 1u : 0u,
+                            int64_t(list.size())};
+      list.resize(list.size() + size_t(m) * width, uint32_t(step.slots) << 16);
+      parallel_ranges(m, [&](int64_t lo, int64_t hi) {
+        for (int64_t l = lo; l < hi; ++l) {
+          const uint32_t p = o[size_t(l)];
+          int64_t to = c.list0 + l;
+          for (size_t t = 0; t < flip.size(); ++t) {
+            if (pc32(p & flip[t]) != 1) continue;
+            const uint32_t src = p ^ flip[t];
+            list[size_t(to)] = at[src] | uint32_t(2 * t + ((src & low[t]) ? 0 : 1)) << 16;
+            to += m;
+          }
+        }
+      });
+      states.insert(states.end(), dep[size_t(r)].begin(), dep[size_t(r)].end());
+      const int32_t each = int32_t(std::max<size_t>(1, share / size_t(m))), count = int32_t(pats[size_t(r)].size());
+      for (int32_t i = 0; i < count; i += each)
+        work.push_back(vqe::GroupWork{int32_t(classes.size()), int32_t(patterns.size()) + i, std::min(each, count - i), 0});
+      patterns.insert(patterns.end(), pats[size_t(r)].begin(), pats[size_t(r)].end());
+      classes.push_back(c);
+    }
+    auto size = [&](const vqe::GroupWork& w) { return w.count * classes[size_t(w.cls)].n; };
+    std::stable_sort(work.begin() + step.work0, work.end(),
+                     [&](const vqe::GroupWork& x, const vqe::GroupWork& y) { return size(x) > size(y); });
+    step.ctas = int32_t(work.size()) - step.work0;
+    if (step.ctas == 0) continue;
+    step.most = size(work[size_t(step.work0)]);
+    plan.steps.push_back(step);
+  }
+  if (work.empty() || vqe::hop_set_limits() != cudaSuccess) {
+    cudaGetLastError();
+    return VQE_OK;
+  }
+  int rc;
+  vqe::HopClass* dc = nullptr;
+  vqe::GroupWork* dw = nullptr;
+  uint32_t *dp = nullptr, *ds = nullptr, *dl = nullptr;
+  int32_t* dt = nullptr;
+  if ((rc = upload_str(e, classes, &dc)) || (rc = upload_str(e, work, &dw)) || (rc = upload_str(e, patterns, &dp)) ||
+      (rc = upload_str(e, states, &ds)) || (rc = upload_str(e, list, &dl)) || (rc = upload_str(e, slots, &dt)))
+    return rc;
+  plan.tables = vqe::HopTables{dc, dw, dp, ds, dl, dt};
+  e->hop = plan;
+  e->use_hop = true;
+  return VQE_OK;
+}
+
 const vqe_hamiltonian_s::Ell* get_ell(vqe_hamiltonian_t h, vqe_ansatz_t a, int* err) {
   *err = VQE_OK;
   std::lock_guard<std::mutex> lock(h->mu);
@@ -1157,6 +1315,13 @@ const vqe_hamiltonian_s::Ell* get_ell(vqe_hamiltonian_t h, vqe_ansatz_t a, int* 
   const double cost = double(D) * double(G);
   if (na >= 0 && G > 0) {
     const int rc = build_strings(h, a, &e);
+    if (rc != VQE_OK) {
+      *err = rc;
+      return nullptr;
+    }
+  }
+  if (na < 0 && G > 0 && !slot_fits(a)) {
+    const int rc = build_hops(h, a, &e);
     if (rc != VQE_OK) {
       *err = rc;
       return nullptr;
@@ -1767,6 +1932,7 @@ vqe::StreamPlan plan(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, cudaStream
   p.n_elec = a->n_elec;
   p.n_alpha = a->n_alpha;
   p.use_ell = e->use_ell;
+  if (e->use_hop && !(g_flags & VQE_FLAG_NO_STRINGS)) p.hop = &e->hop;
   p.use_str = e->use_str && !(g_flags & VQE_FLAG_NO_STRINGS);
   p.str = e->str;
   p.use_tc = p.use_str && e->use_tc;
@@ -1989,6 +2155,7 @@ int prepare_noalloc(vqe_hamiltonian_s* h, vqe_ansatz_s* a, bool with_grad, size_
   *d = make_desc(h, a, e, 0);
   *sp = plan(a, e, nullptr, false);
   sp->use_tc = false;  // its operands do not fit the scratch
+  sp->hop = nullptr;   // nor do its tables
   sp->sweep = nullptr;  // one launch per gate: the sweep queues address the regular workspace layout
   // the string-driven H psi needs two more sector-sized vectors; when they do
   // not fit, the connectivity rows (if built) or the group scan serve instead

@@ -398,6 +398,40 @@ cudaError_t group_forward(const InstDesc& d, const GroupPlan& p, const GroupBuff
 cudaError_t group_reverse(const InstDesc& d, const GroupPlan& p, const GroupBuffers& w, const double* psi,
                           const double* lam, void* scratch, double* grad, cudaStream_t stream);
 
+// H psi of a large electron-number sector by hops (vqe_hop.cu).
+constexpr int kHopStates = 12928;    // amplitudes per CTA: two CTAs per SM
+constexpr int kHopSlots = 512;       // hop values of a pass (two directions each)
+struct HopClass {            // blocks of a pass with the same electron count on its qubits
+  int32_t n, state0, width;  // local states states[state0 ...], entries per state
+  uint32_t inv;              // 2^32 / n, rounded up
+  int64_t list0;             // entry e of state l: list[list0 + e n + l] = source state | value << 16
+};
+struct HopTables {
+  const HopClass* classes;
+  const GroupWork* work;     // the largest first
+  const uint32_t* patterns;  // occupations of the other qubits
+  const uint32_t* states;
+  const uint32_t* list;      // value s.slots: 0 (padding)
+  const int32_t* slots;      // table slot of each value
+};
+struct HopStep {             // one pass
+  int32_t work0, ctas, most, slot0, slots;
+};
+struct HopDiag {             // the diagonal group: first slot (-1: none), row stride, counted qubits
+  int32_t slot, stride;
+  uint32_t counted;
+};
+struct HopPlan {
+  HopTables tables{};
+  HopDiag diag{};
+  std::vector<HopStep> steps;
+};
+int hop_width(int w);        // entries per state, rounded up as the kernel reads them
+cudaError_t hop_set_limits();
+// lambda = H psi; tab: (2 + high-half qubits) 2^lo_bits doubles
+cudaError_t hop_hpsi(const InstDesc& d, const HopPlan& p, double* tab, const double* psi, double* lam,
+                     cudaStream_t stream);
+
 struct StreamBuffers {
   void* psi = nullptr;     // D amplitudes (double or double2), sector order
   void* lam = nullptr;     // D amplitudes
@@ -462,6 +496,7 @@ struct StreamPlan {
   bool use_ell;
   bool use_str;                  // string-driven H psi with `str`
   StrPlan str;
+  const HopPlan* hop = nullptr;  // real amplitudes: H psi by hops
   bool use_tc = false;           // real amplitudes: tc, and rest for the groups outside it
   bool has_rest = false;
   TcPlan tc;

@@ -928,6 +928,11 @@ cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuf
     }
     k_perm_scatter<REAL><<<grid, kStreamThreads, 0, stream>>>(sp.str.perm, d.D, lam_am, lam);
     k_dot<REAL><<<grid, kStreamThreads, 0, stream>>>(psi, lam, d.D, b.epart);
+  } else if (REAL && sp.hop) {
+    const cudaError_t e = hop_hpsi(d, *sp.hop, static_cast<double*>(b.psi_am), static_cast<const double*>(b.psi),
+                                   static_cast<double*>(b.lam), stream);
+    if (e != cudaSuccess) return e;
+    k_dot<REAL><<<grid, kStreamThreads, 0, stream>>>(psi, lam, d.D, b.epart);
   } else if (sp.use_ell) {
     k_hpsi<REAL, true><<<grid, kStreamThreads, 0, stream>>>(d, sp.n_elec, sp.n_alpha, psi, lam, b.epart);
   } else {

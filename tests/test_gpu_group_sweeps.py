@@ -1,5 +1,6 @@
 """The gate sweeps by groups (csrc/vqe_group.cu) against the launches per gate
-(VQE_FLAG_FP64_SWEEPS): spin and electron-number sectors, low and odd electron
+(VQE_FLAG_FP64_SWEEPS), and H psi by hops (csrc/vqe_hop.cu) against the connectivity
+rows (VQE_FLAG_NO_STRINGS): spin and electron-number sectors, low and odd electron
 counts, one gate, repeated gates and gates that no state allows.
 
 Tolerance: fixed point keeps 2^-62 of the norm per rotation and 2^-61 ||lambda|| per
@@ -58,3 +59,5 @@ def test_number_sectors(n, pairs, gates):
     (e, g, only), (e1, g1, _) = _both(H, A, th, vq.VQE_FLAG_FP64_SWEEPS)
     assert only == e
     assert abs(e - e1) <= 1e-10 and float((g - g1).abs().max()) <= 1e-10
+    (_, _, _), (e2, g2, _) = _both(H, A, th, vq.VQE_FLAG_NO_STRINGS)
+    assert abs(e - e2) <= 1e-10 and float((g - g2).abs().max()) <= 1e-10
