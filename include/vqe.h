@@ -33,7 +33,9 @@
  * synchronously, and the pair keeps them until the Hamiltonian is destroyed.
  * Under VQE_FLAG_PERSISTENT_SWEEPS the first streaming evaluation of an ansatz
  * (or vqe_workspace_bytes with it) also builds the task queues of its
- * persistent gate sweeps. After that the compute calls allocate nothing, so
+ * persistent gate sweeps. The first evaluation of an ansatz on a large sector (or
+ * vqe_workspace_bytes with it, or a batch's creation) builds the tables of its gate
+ * groups; under stream capture it does not, and runs a launch per gate. After that the compute calls allocate nothing, so
  * make those first calls before any stream capture. Every compute call is asynchronous on the given
  * stream (a cudaStream_t; NULL is the legacy default stream) except where
  * noted.
@@ -78,9 +80,10 @@ int vqe_version(void);
  *   VQE_FLAG_FORCE_STREAMING never use the shared-memory-resident kernel;
  *   VQE_FLAG_NO_CLUSTER      run each resident instance on one CTA instead of
  *                            a cluster of two;
- *   VQE_FLAG_FP64_SWEEPS     run the resident kernel's gate sweeps in FP64
- *                            instead of 64-bit fixed point (H psi, the energy
- *                            and every streaming kernel are FP64 either way);
+ *   VQE_FLAG_FP64_SWEEPS     run the gate sweeps in FP64 instead of 64-bit fixed
+ *                            point: in the resident kernel, and with a launch
+ *                            per gate (or VQE_FLAG_PERSISTENT_SWEEPS) where they
+ *                            run in cluster shared memory or by groups of gates;
  *   VQE_FLAG_NO_STRINGS      streaming H psi by connectivity rows (or a scan of
  *                            all groups) instead of alpha/beta strings;
  *   VQE_FLAG_PERSISTENT_SWEEPS streaming gate sweeps of a single instance as
@@ -88,7 +91,8 @@ int vqe_version(void);
  *                            instead of one launch per gate; the same bits as
  *                            one launch per gate without the kept forward
  *                            outputs (below), and slower on the GPUs measured
- *                            (kept for comparison);
+ *                            (kept for comparison; sweeps in cluster shared
+ *                            memory or by groups are not affected);
  *   VQE_FLAG_NO_PHI_STORE    real instances of 6,000,000 sector states or more
  *                            normally keep the forward sweep's outputs of every
  *                            amplitude pair in the workspace (16 bytes per pair)
