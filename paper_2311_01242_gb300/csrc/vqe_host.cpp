@@ -1738,6 +1738,7 @@ struct GroupBuild {
   std::vector<uint32_t> patterns, states, pairs;
   int most = 0, most_pairs = 0;
 };
+constexpr int kGroupQubits = 20;  // build_group lists every occupation of them (few electrons of one spin leave few states)
 // The most ways, over the electron counts r that s of n qubits can hold of k, to place
 // r - f / 2 electrons on s - f qubits: local states (f = 0), or pairs of a gate that
 // flips f qubits.
@@ -1754,6 +1755,7 @@ bool group_fits(vqe_ansatz_t a, uint32_t set, const std::vector<int>& gates) {
     return most_ways(sa, a->n_alpha, na, pc32(flip & even)) *
            most_ways(sb, a->n_elec - a->n_alpha, nb, pc32(flip & ~even));
   };
+  if (pc32(set) > kGroupQubits) return false;
   size_t pairs = 0;
   for (int m : gates) pairs += ways(a->gates[size_t(m)].flip);
   return pairs <= size_t(vqe::kGroupPairs) && std::min(ways(0), 2 * pairs) <= size_t(vqe::kGroupStates) &&
