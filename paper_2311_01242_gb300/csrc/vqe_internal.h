@@ -129,9 +129,10 @@ struct TcScratch {
   int* vexp;                 // [items]
   int* vodd;                 // [items]
   double* vsum;              // [items]
+  int4* row;                 // [Da] scales of an output row: ea, e, de, flags (bad | odd << 1)
 };
 struct TcOffsets {           // the same as byte offsets from the workspace's start, and the
-  int64_t dig, one_a, one_b, pexp, aexp, ade, bexp, bde, vi, vexp, vodd, vsum;
+  int64_t dig, one_a, one_b, pexp, aexp, ade, bexp, bde, vi, vexp, vodd, vsum, row;
   int64_t psi_am, lam_am;    // alpha-major source and result (unsigned, FP64)
 };
 struct TcInst {

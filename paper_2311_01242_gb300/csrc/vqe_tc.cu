@@ -222,6 +222,7 @@ __device__ __forceinline__ TcScratch scratch_of(const TcInst& I, char* ws) {
   s.vexp = reinterpret_cast<int*>(ws + I.off.vexp);
   s.vodd = reinterpret_cast<int*>(ws + I.off.vodd);
   s.vsum = reinterpret_cast<double*>(ws + I.off.vsum);
+  s.row = reinterpret_cast<int4*>(ws + I.off.row);
   return s;
 }
 
@@ -342,7 +343,7 @@ __global__ void __launch_bounds__(256) k_tc_digits(const TcInst* __restrict__ ma
 struct TcShared {          // after the operand buffers and the lambda row
   uint64_t full[kMaxStages], empty[kMaxStages], tfull, tempty, last;
   uint32_t tmem;
-  int dead, bad, odd, ea, shift_hi, shift_lo, e;
+  int dead, bad, odd, shift_hi, shift_lo, e;
   uint32_t src[kChunkK];   // source row
   int32_t item[kChunkK];
   int32_t sh[kChunkK];     // shift of the item's values | sign << 16
@@ -406,51 +407,15 @@ k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int
     double* lam_am = reinterpret_cast<double*>(ws + I.off.lam_am);
     const int R = tc.MT * kRows;  // entries of dst hold eight strings
     const int n_tiles = tc.DbP / kTileN;
-    // scales of this row: 2^ea above every |V psi'| element, 2^e above every partial sum of lambda'
-    if (warp == 0) {
-      int top = -100000, bad = 0, odd = 0;
-      for (int k = lane; k < tc.K; k += 32) {
-        const uint32_t kj = __ldg(tc.kj + int64_t(ia) * tc.KT + k);
-        const int it = __ldg(tc.kit + int64_t(ia) * tc.KT + k);
-        const int ve = __ldg(sc.vexp + it), pe = __ldg(sc.pexp + (kj & 0x7fffffffu));
-        bad |= ve == kBadExp || pe == kBadExp;
-        odd |= __ldg(sc.vodd + it);
-        top = max(top, ve + pe);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-        odd |= __shfl_xor_sync(0xffffffffu, odd, o);
-      }
-      double sum = 0.0;
-      if (!bad)
-        for (int k = lane; k < tc.K; k += 32) {
-          const uint32_t kj = __ldg(tc.kj + int64_t(ia) * tc.KT + k);
-          const int it = __ldg(tc.kit + int64_t(ia) * tc.KT + k);
-          const int d = __ldg(sc.vexp + it) + __ldg(sc.pexp + (kj & 0x7fffffffu)) - top;  // <= 0
-          // vsum <= 2 R 2^vexp: its mantissa against the item's own scale
-          if (d > -200) sum += ldexp(__ldg(sc.vsum + it), d - __ldg(sc.vexp + it));
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (lane == 0) {
-        const int de = max(1, exp_above(sum * 1.0000001));
-        S.ea = top;
-        S.e = top + de;
-        S.shift_hi = 28 - de;
-        S.shift_lo = de - 1;
-        S.bad = bad;
-        S.odd = odd;
-      }
+    const int4 scales = __ldg(sc.row + ia);
+    if (tid == 0) {
+      S.e = scales.y;
+      S.shift_hi = 28 - scales.z;
+      S.shift_lo = scales.z - 1;
+      S.bad = scales.w & 1;
+      S.odd = scales.w >> 1;
     }
-    for (int j = tid; j < tc.DbP; j += kThreads) lam_lo[j] = lam_hi[j] = 0u;
-    __syncthreads();
-    const int passes = S.bad ? 0 : tc.MT * tc.chunks * (S.odd ? 2 : 1);
-    for (int ps = 0; ps < passes; ++ps) {
-      const int kc = ps % tc.chunks, mt = (ps / tc.chunks) % tc.MT, od = ps / (tc.chunks * tc.MT);
-      const int kcnt = min(kChunkK, tc.K - kc * kChunkK);
-      const int ksteps = (kcnt + 15) >> 4;
+    auto sources = [&](int kc) {  // of one chunk
       if (tid < kChunkK) {
         const int64_t q = int64_t(ia) * tc.KT + kc * kChunkK + tid;
         const uint32_t kj = __ldg(tc.kj + q);
@@ -458,9 +423,21 @@ k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int
         const uint32_t r = kj & 0x7fffffffu;
         S.src[tid] = r;
         S.item[tid] = it;
-        S.sh[tid] = min(S.ea - __ldg(sc.vexp + it) - __ldg(sc.pexp + r), 63) | int((kj >> 31) << 16);
+        S.sh[tid] = min(scales.x - __ldg(sc.vexp + it) - __ldg(sc.pexp + r), 63) | int((kj >> 31) << 16);
       }
-      __syncthreads();
+    };
+    sources(0);
+    for (int j = tid; j < tc.DbP; j += kThreads) lam_lo[j] = lam_hi[j] = 0u;
+    __syncthreads();
+    const int passes = S.bad ? 0 : tc.MT * tc.chunks * (S.odd ? 2 : 1);
+    for (int ps = 0; ps < passes; ++ps) {
+      const int kc = ps % tc.chunks, mt = (ps / tc.chunks) % tc.MT, od = ps / (tc.chunks * tc.MT);
+      const int kcnt = min(kChunkK, tc.K - kc * kChunkK);
+      const int ksteps = (kcnt + 15) >> 4;
+      if (ps > 0) {
+        sources(kc);
+        __syncthreads();
+      }
       // A: digits of V times the sources' scales, [digit][hop][k], 16 bytes (8 k) at a time
       const long long* vi = sc.vi + int64_t(od) * tc.items * R + mt * kRows;
       for (int q = tid; q < kRows * 2 * ksteps; q += kThreads) {
@@ -626,6 +603,42 @@ k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int
 }
 
 // ---------------------------------------------------------------- one-spin part
+// Scales of output row ia of the product kernel, by one warp: 2^ea above every |V psi'|
+// element, 2^e = 2^(ea + de) above every partial sum of lambda'. (Here, beside the row of
+// the alpha matrix, four loads' latency passes for all rows at once; in the product kernel
+// it passed row by row: H psi of 26 qubits and 11 electrons 2.93 -> 2.87 ms, 24 qubits energy
+// and gradient 1.90 -> 1.87 ms.)
+__device__ __forceinline__ int4 row_scales(const TcPlan& tc, const TcScratch& sc, int ia, int lane) {
+  int top = -100000, bad = 0, odd = 0;
+  for (int k = lane; k < tc.K; k += 32) {
+    const uint32_t kj = __ldg(tc.kj + int64_t(ia) * tc.KT + k);
+    const int it = __ldg(tc.kit + int64_t(ia) * tc.KT + k);
+    const int ve = __ldg(sc.vexp + it), pe = __ldg(sc.pexp + (kj & 0x7fffffffu));
+    bad |= ve == kBadExp || pe == kBadExp;
+    odd |= __ldg(sc.vodd + it);
+    top = max(top, ve + pe);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+    odd |= __shfl_xor_sync(0xffffffffu, odd, o);
+  }
+  double sum = 0.0;
+  if (!bad)
+    for (int k = lane; k < tc.K; k += 32) {
+      const uint32_t kj = __ldg(tc.kj + int64_t(ia) * tc.KT + k);
+      const int it = __ldg(tc.kit + int64_t(ia) * tc.KT + k);
+      const int d = __ldg(sc.vexp + it) + __ldg(sc.pexp + (kj & 0x7fffffffu)) - top;  // <= 0
+      // vsum <= 2 R 2^vexp: its mantissa against the item's own scale
+      if (d > -200) sum += ldexp(__ldg(sc.vsum + it), d - __ldg(sc.vexp + it));
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  const int de = max(1, exp_above(sum * 1.0000001));
+  return make_int4(top, top + de, de, bad | odd << 1);
+}
+
 // Digits of one row of a one-spin matrix (H's terms that move electrons of one
 // spin only, and that spin's diagonal): row r as a dense vector of n values, each
 // the sum of its table slots, times 2^fold[col] (the source rows' exponents; null:
@@ -648,6 +661,10 @@ __global__ void __launch_bounds__(256) k_tc_onespin(const TcInst* __restrict__ m
   const int r = blockIdx.x, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   for (int j = tid; j < ld; j += blockDim.x) srow[j] = 0.0;
   __syncthreads();
+  if (!beta && w == 7) {
+    const int4 scales = row_scales(I.tc, sc, r, lane);
+    if (lane == 0) sc.row[r] = scales;
+  }
   const int e0 = __ldg(os.off + r), e1 = __ldg(os.off + r + 1);
   int top = -100000;
   for (int e = e0 + tid; e < e1; e += blockDim.x) {
