@@ -41,9 +41,18 @@ def _ptr(a):
     return a.ctypes.data
 
 
+# The current stream's handle without the Stream object: torch.cuda.current_stream() takes 8
+# of the 24 us that the smallest call (4 qubits, a 10 us kernel) cost the host
+# (27.5 -> 20.0 us a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def set_flags(flags: int) -> int:
