@@ -3276,8 +3276,15 @@ static int build_mid_batch(vqe_batch_s* B) {
       k.threads = std::max(k.threads, shape[size_t(i)].threads);
       ++k.n;
     }
-    for (size_t j = first.back(); j < sweep.size(); ++j)
-      k.smem = std::max(k.smem, vqe::sweep_smem(sweep[j].M, c, sweep[j].shift, sweep[j].D, k.threads));
+    // the most threads that any of the class wants, but no more than fit beside every state
+    // (each instance fits with its own, and results do not depend on them)
+    for (;; k.threads /= 2) {
+      k.smem = 0;
+      for (size_t j = first.back(); j < sweep.size(); ++j)
+        k.smem = std::max(k.smem, vqe::sweep_smem(sweep[j].M, c, sweep[j].shift, sweep[j].D, k.threads));
+      if (k.smem + 1024 <= optin || k.threads <= 128) break;
+    }
+    if (k.smem + 1024 > optin) return fail(VQE_ERR_UNSUPPORTED, "sweeps of the batch do not fit shared memory");
     if (k.n > 0)
       sb.classes.push_back(k);
     else
