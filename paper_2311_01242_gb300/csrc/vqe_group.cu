@@ -17,7 +17,7 @@
 // at 24 qubits; 2.7 million boson states and 144 gates 4.3 -> 2.2 ms. Issue slots
 // bound the gates of large sectors, latencies the rest. The reverse sweep un-applies psi
 // beside lambda ({psi, lambda} as 16 bytes), so no forward outputs are kept; gradient
-// sums are integers: exact and independent of the order of blocks. Tried: 256 threads per
+// sums are integers: exact and independent of the order of blocks (cross_add). Tried: 256 threads per
 // CTA (24 qubits 8 % slower), 608 CTAs (10 % slower, nothing of the next launch fits
 // beside them), 5,120 amplitudes per CTA (boson sector 10 % slower), pair lists read
 // from L2 gate by gate (a latency per gate).
@@ -61,7 +61,7 @@ k_group_init(int64_t D, int64_t hf_rank, int M, const int64_t* __restrict__ pair
   }
   for (int64_t r = i0; r < D; r += step) psi[r] = r == hf_rank ? 1ll << 62 : 0ll;
   if (gacc)
-    for (int64_t r = i0; r < int64_t(M) * kGroupCopies; r += step) gacc[r] = 0ull;
+    for (int64_t r = i0; r < int64_t(M) * 2 * kGroupCopies; r += step) gacc[r] = 0ull;
 }
 
 struct GateShared {
@@ -79,6 +79,7 @@ k_group_gates(const GroupTables T, const GroupStep s, long long* __restrict__ v,
   __shared__ GateShared gate[kGroupGates];
   __shared__ uint32_t sign[kGroupPatterns];  // of each block, a bit per gate
   __shared__ long long part[REV ? kGroupGates * kWarps : 1];
+  __shared__ uint32_t part_lo[REV ? kGroupGates * kWarps : 1];
   longlong2* st2 = reinterpret_cast<longlong2*>(st);
   uint32_t* pairs = reinterpret_cast<uint32_t*>(st + size_t(s.most) * (REV ? 2 : 1));
   uint32_t* rank = pairs + s.most_pairs;
@@ -140,7 +141,7 @@ k_group_gates(const GroupTables T, const GroupStep s, long long* __restrict__ v,
   const int g0 = REV ? s.gates - 1 : 0, step = REV ? -1 : 1;
   GateShared t = gate[g0];
   for (int k = 0; k < s.gates; ++k) {
-    long long acc = 0;
+    CrossSum acc{0, 0u};
     const int n = t.n * w.count, g = g0 + k * step;
     const int nh = -t.sh, nl = -t.sl;
 #pragma unroll 1
@@ -155,7 +156,7 @@ k_group_gates(const GroupTables T, const GroupStep s, long long* __restrict__ v,
         const Words a = split(va.x), b = split(vb.x), la = split(va.y), lb = split(vb.y);
         st2[ia] = make_longlong2(turn(a, b, t.ch, t.cl, t.sh, t.sl), turn(la, lb, t.ch, t.cl, t.sh, t.sl));
         st2[ib] = make_longlong2(turn(b, a, t.ch, t.cl, nh, nl), turn(lb, la, t.ch, t.cl, nh, nl));
-        acc += cross_high(a, lb, b, la);
+        cross_add(acc, a, lb, b, la, false);
       } else {
         const Words a = split(st[ia]), b = split(st[ib]);
         st[ia] = turn(a, b, t.ch, t.cl, nh, nl);
@@ -164,16 +165,11 @@ k_group_gates(const GroupTables T, const GroupStep s, long long* __restrict__ v,
     }
     if (k + 1 < s.gates) t = gate[g + step];
     if (REV) {
-      // the warp's sum in three pieces of 24, 24 and 16 bits (each fits 32 after 32 lanes)
-      long long r = 0;
-      if ((tid & ~31) < n) {
-        const uint32_t s0 = __reduce_add_sync(0xffffffffu, uint32_t(acc) & 0xffffffu);
-        const uint32_t s1 = __reduce_add_sync(0xffffffffu, uint32_t(acc >> 24) & 0xffffffu);
-        const int s2 = __reduce_add_sync(0xffffffffu, int(acc >> 48));
-        r = static_cast<long long>(s0) + (static_cast<long long>(s1) << 24) +
-            static_cast<long long>(static_cast<uint64_t>(static_cast<long long>(s2)) << 48);
+      if ((tid & ~31) < n) acc = cross_warp(acc);
+      if (lane == 0) {
+        part[g * kWarps + warp] = acc.hi;
+        part_lo[g * kWarps + warp] = acc.lo;
       }
-      if (lane == 0) part[g * kWarps + warp] = r;
     }
     if (n > 0) __syncthreads();
   }
@@ -181,9 +177,15 @@ k_group_gates(const GroupTables T, const GroupStep s, long long* __restrict__ v,
     __syncthreads();
     if (tid < s.gates && range.y > 0) {
       long long r = 0;
+      unsigned long long lo = 0;
 #pragma unroll
-      for (int i = 0; i < kWarps; ++i) r += part[tid * kWarps + i];
-      atomicAdd(gacc + int64_t(blockIdx.x % kGroupCopies) * M + rec.m, static_cast<unsigned long long>(r));
+      for (int i = 0; i < kWarps; ++i) {
+        r += part[tid * kWarps + i];
+        lo += part_lo[tid * kWarps + i];
+      }
+      unsigned long long* to = gacc + int64_t(blockIdx.x % kGroupCopies) * 2 * M + rec.m;
+      atomicAdd(to, static_cast<unsigned long long>(r));
+      atomicAdd(to + M, lo);
     }
   }
   if (!store) return;
@@ -239,12 +241,15 @@ k_group_final(const unsigned long long* __restrict__ gacc, int M, const double* 
               double* __restrict__ grad) {
   const int m = blockIdx.x * kStreamThreads + threadIdx.x;
   if (m >= M) return;
-  unsigned long long v = 0;
+  unsigned long long v = 0, lo = 0;
 #pragma unroll 8
-  for (int i = 0; i < kGroupCopies; ++i) v += gacc[int64_t(i) * M + m];
+  for (int i = 0; i < kGroupCopies; ++i) {
+    v += gacc[int64_t(2 * i) * M + m];
+    lo += gacc[int64_t(2 * i + 1) * M + m];
+  }
   const double n2 = *l2;
   grad[m] = n2 < llbits(0x7ff0000000000000ll)
-                ? __ll2double_rn(static_cast<long long>(v)) * pow2(norm_exp(n2) - 61)
+                ? cross_value(static_cast<long long>(v), lo) * pow2(norm_exp(n2) - 61)
                 : llbits(0x7ff8000000000000ll);
 }
 

@@ -1617,7 +1617,7 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   L.sw_phi = L.sw_gacc = L.sw_dot = 0;
   if (L.has_tc && mid_ansatz(a)) {
     L.sw_gacc = L.total;
-    L.sw_dot = L.sw_gacc + align256(size_t(std::max(a->M, 1)) * 8);
+    L.sw_dot = L.sw_gacc + align256(size_t(std::max(a->M, 1)) * 16);
     L.sw_phi = L.sw_dot + align256(size_t(2 * vqe::kSweepDots) * 8);
     L.total = L.sw_phi + (with_grad ? align256(std::max<size_t>(a->pairs.size(), 1) * 16) : 0);
   }
@@ -1626,7 +1626,7 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
     L.gr_norm = L.total;
     L.gr_trig = L.gr_norm + align256(size_t(vqe::kMaxPartials + 2) * 8);
     L.gr_gacc = L.gr_trig + align256(size_t(a->M) * 16);
-    L.total = L.gr_gacc + (with_grad ? align256(size_t(a->M) * vqe::kGroupCopies * 8) : 0);
+    L.total = L.gr_gacc + (with_grad ? align256(size_t(a->M) * vqe::kGroupCopies * 16) : 0);
   }
   return L;
 }

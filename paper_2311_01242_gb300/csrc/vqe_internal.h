@@ -387,7 +387,7 @@ struct GroupPlan {
 };
 struct GroupBuffers {
   int4* trig;                // [M]
-  unsigned long long* gacc;  // [kGroupCopies][M]
+  unsigned long long* gacc;  // [kGroupCopies][high and low part][M]
   double* norm;              // <lambda|lambda>, then kMaxPartials partial sums of it
   int* bad;
 };
