@@ -34,11 +34,11 @@
  * Under VQE_FLAG_PERSISTENT_SWEEPS the first streaming evaluation of an ansatz
  * (or vqe_workspace_bytes with it) also builds the task queues of its
  * persistent gate sweeps. The first evaluation of an ansatz on a large sector (or
- * vqe_workspace_bytes with it, or a batch's creation) builds the tables of its gate
- * groups; under stream capture it does not, and runs a launch per gate. After that the compute calls allocate nothing, so
- * make those first calls before any stream capture. Every compute call is asynchronous on the given
- * stream (a cudaStream_t; NULL is the legacy default stream) except where
- * noted.
+ * vqe_workspace_bytes or vqe_pool_workspace_bytes with it, or a batch's creation) builds
+ * the tables of its gate groups; under stream capture it does not, and runs a launch per
+ * gate. After that the compute calls allocate nothing, so make those first calls before
+ * any stream capture. Every compute call is asynchronous on the given stream (a
+ * cudaStream_t; NULL is the legacy default stream) except where noted.
  *
  * Errors: every int-returning call returns VQE_OK (0) or a VQE_ERR_* code and
  * sets a thread-local message readable with vqe_last_error(). Invalid

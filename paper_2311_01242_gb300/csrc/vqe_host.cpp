@@ -2945,6 +2945,7 @@ size_t vqe_pool_workspace_bytes(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_ansatz_
   int rc = VQE_OK;
   if (!get_ell(h, a, &rc)) return 0;
   const bool real = use_real();
+  if (real && group_ansatz(a)) get_groups(a, nullptr);  // as vqe_workspace_bytes
   return ws_layout(a, !real, false).total + align256(size_t(std::max<int64_t>(pool->chunk_off.back(), 1)) * 8) +
          align256(std::max<size_t>(a->sector.size(), 1) * (real ? 16 : 32));
 }
