@@ -1563,11 +1563,16 @@ bool mid_ansatz(vqe_ansatz_t a) {
 // Whether the gate sweeps of this ansatz can run in groups (get_groups). A gate of a spin
 // sector touches an eighth of the amplitudes at most, a group of a few gates half of
 // them: from a few million states on, where launches no longer count, a launch per gate
-// moves less.
-constexpr int64_t kGroupSpinStates = int64_t(3) << 19;
+// moves less. A fixed-point rotation rounds at 2^-62 of the norm whatever the amplitude, so the
+// state's error grows with the square root of the states, FP64's does not: against long
+// double, with random angles of 0.4, 2.7 million boson states and 144 gates 4.9e-16 against
+// 6.4e-16, 4.5 million 6.1e-16 against 6.6e-16, 5.2 million 6.2e-16 against 6.0e-16, 10.4
+// million 7.8e-16 against 6.3e-16. Above the bound sweeps are FP64 (5.2 million states: energy
+// and gradient 10.6 ms, by groups 8.0 ms).
+constexpr int64_t kGroupSpinStates = int64_t(3) << 19, kGroupNumberStates = int64_t(1) << 22;
 bool group_ansatz(vqe_ansatz_t a) {
   const int64_t D = int64_t(a->sector.size());
-  return !a->pairs.empty() && D > kSweepStates && (a->n_alpha < 0 || D <= kGroupSpinStates);
+  return !a->pairs.empty() && D > kSweepStates && D <= (a->n_alpha < 0 ? kGroupNumberStates : kGroupSpinStates);
 }
 
 WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
