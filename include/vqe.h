@@ -406,27 +406,33 @@ int vqe_batch_energy_grad_host(vqe_batch_t b, const double* theta_host, int64_t 
  * resident instances (a multiple of 32 in [32, 512]; 0 keeps the current
  * value). Rebuilds the task queues; synchronous. Results do not depend on any
  * of them. vqe_batch_get_tuning reports the current values, the persistent
- * grid and the task count of the gradient queue (any output may be NULL).
+ * grid (without persistent instances the CTAs of the cluster sweeps) and the number
+ * of tasks with the gradient, as vqe_batch_set_wait counts them (any output may be NULL).
  */
 int vqe_batch_set_tuning(vqe_batch_t b, int ctas_per_sm, int gate_chunk, int sweep_threads);
 int vqe_batch_get_tuning(vqe_batch_t b, int* ctas_per_sm, int* gate_chunk, int* grid, int64_t* n_tasks);
 
 /*
- * Bounded waits of the persistent launch. A CTA whose task depends on
- * unfinished tasks of the same instance polls that instance's progress counter
- * for at most budget_ns nanoseconds (default 2e9; 1e3 .. 6e11 accepted), then
+ * Bounded waits of the batch's launches. A CTA of the persistent launch whose task
+ * depends on unfinished tasks of the same instance polls that instance's progress
+ * counter for at most budget_ns nanoseconds (default 2e9; 1e3 .. 6e11 accepted), then
  * writes its task's index + 1 into the status word in the workspace, takes no
- * more tasks and returns; the other CTAs stop at their next task or wait, and
- * every energy and gradient of the persistent instances is written as NaN.
+ * more tasks and returns; the other CTAs stop at their next task or wait. The
+ * tensor-core H psi of the instances swept in cluster shared memory waits for its own
+ * copies and products for two seconds at most and reports in the same way. Then every
+ * energy and gradient of the persistent and of the swept instances is written as NaN;
+ * resident instances and those evaluated one by one keep theirs.
  * vqe_batch_energy_grad_host then returns VQE_ERR_TIMEOUT; after the device
- * call, vqe_batch_status does. probe_task >= 0 makes that task of the queue
- * wait for a count that no task reaches, so its wait runs out (a check of the
- * timeout path that stops no GPU); -1 for normal operation.
+ * call, vqe_batch_status does. probe_task >= 0 makes that task wait for something
+ * that nothing reaches, so its wait runs out (a check of the timeout path that stops
+ * no GPU): tasks are the queue's, then one for each instance's forward sweep, one for
+ * each reverse sweep and one for their H psi. -1 for normal operation. (In calls
+ * without a batch a wait of the tensor-core H psi that runs out makes the result NaN.)
  */
 int vqe_batch_set_wait(vqe_batch_t b, int64_t budget_ns, int32_t probe_task);
 
 /*
- * Status of the last persistent launch that used `workspace` (the batch's
+ * Status of the last batch call that used `workspace` (the batch's
  * workspace as passed to vqe_batch_energy_grad): synchronises `stream`, reads
  * the status word, and returns VQE_OK or VQE_ERR_TIMEOUT (the message names the
  * task and instance whose wait ran out).

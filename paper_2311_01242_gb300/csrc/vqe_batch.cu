@@ -363,14 +363,14 @@ cudaError_t persistent_sweep_run(const PersistDev& p, int grid, const double* th
   return cudaGetLastError();
 }
 
-cudaError_t batch_persistent_run(const PersistDev& p, int grid, size_t smem, const PFinal* rows, int n_rows,
-                                 int n_grad_rows, const double* theta, int64_t ld_theta, double* energy, double* grad,
-                                 int64_t ld_grad, cudaStream_t stream) {
-  cudaError_t e = cudaMemsetAsync(p.counters, 0, size_t(p.n + 2) * sizeof(int), stream);
-  if (e != cudaSuccess) return e;
+cudaError_t batch_persistent_run(const PersistDev& p, int grid, size_t smem, const double* theta, int64_t ld_theta,
+                                 cudaStream_t stream) {
   k_batch_persistent<<<grid, kPersistThreads, smem, stream>>>(p, theta, ld_theta);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t batch_persistent_final(const PersistDev& p, const PFinal* rows, int n_rows, int n_grad_rows,
+                                   double* energy, double* grad, int64_t ld_grad, cudaStream_t stream) {
   // gradient rows come first; without a gradient only the energy rows run
   const PFinal* r0 = grad ? rows : rows + n_grad_rows;
   const int nr = grad ? n_rows : n_rows - n_grad_rows;

@@ -2104,7 +2104,7 @@ int run_mid(vqe_hamiltonian_t h, vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e
   const vqe::SweepCtl ctl{nullptr, nullptr, 0, -1, 0, 0};
   const vqe::TcInst T = tc_inst(h, e, L, 0);
   cudaError_t ce = vqe::sweep_forward(k, &I, ws, theta, 0, grad != nullptr, ctl, stream);
-  if (ce == cudaSuccess) ce = vqe::tc_hpsi(vqe::tc_single(e->tc), &T, ws, false, stream);
+  if (ce == cudaSuccess) ce = vqe::tc_hpsi(vqe::tc_single(e->tc), &T, ws, false, vqe::TcCtl{}, stream);
   if (ce == cudaSuccess) ce = vqe::sweep_dots(nullptr, &I, 1, ws, stream);
   if (ce == cudaSuccess && grad) ce = vqe::sweep_reverse(k, &I, ws, theta, 0, ctl, stream);
   if (ce == cudaSuccess) ce = vqe::sweep_final(nullptr, &I, 1, ws, theta, 0, ctl, energy, grad, 0, stream);
@@ -3487,9 +3487,9 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
     int queued = 0;
     cudaError_t ce = cudaMemsetAsync(counters, 0, size_t(n_slots + 3) * sizeof(int), stream);
     if (ce != cudaSuccess) return cuda_fail(ce, "batch counters");
+    vqe::PersistDev pd;
     if (n_slots > 0) {
       const PersistQueue& Q = *sb.q[with_grad ? 1 : 0];
-      vqe::PersistDev pd;
       pd.desc = sb.d_desc;
       pd.slots = sb.d_slots;
       pd.tasks = Q.d_tasks;
@@ -3501,18 +3501,30 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
       pd.probe_task = sb.probe_task;
       pd.pad = 0;
       if ((rc = ensure_persist_smem(sb.smem))) return rc;
-      ce = vqe::batch_persistent_run(pd, sb.grid, sb.smem, Q.d_finals, int(Q.finals.size()), Q.n_grad_rows, theta,
-                                     ld_theta, energies, with_grad ? grads : nullptr, ld_grad, stream);
+      ce = vqe::batch_persistent_run(pd, sb.grid, sb.smem, theta, ld_theta, stream);
       if (ce != cudaSuccess) return cuda_fail(ce, "persistent batch launch");
     }
+    // outputs last: a wait of either kind that runs out makes all of them NaN
+    auto finish_slots = [&]() -> int {
+      if (n_slots == 0) return VQE_OK;
+      const PersistQueue& Q = *sb.q[with_grad ? 1 : 0];
+      const cudaError_t fe = vqe::batch_persistent_final(pd, Q.d_finals, int(Q.finals.size()), Q.n_grad_rows, energies,
+                                                         with_grad ? grads : nullptr, ld_grad, stream);
+      return fe == cudaSuccess ? VQE_OK : cuda_fail(fe, "persistent batch outputs");
+    };
     if (!sb.mid.empty() && mid_flags()) {
       char* w = static_cast<char*>(ws);
       const int n = int(sb.mid.size());
       const vqe::SweepCtl ctl{counters + n_slots + 1, counters + n_slots + 2, sb.budget_ns, sb.probe_task, queued, n};
+      vqe::TcCtl tctl;
+      tctl.status = ctl.status;
+      tctl.code = queued + 2 * n + 1;
+      tctl.probe = sb.probe_task == queued + 2 * n;
+      tctl.budget_ns = sb.budget_ns;
       ce = cudaSuccess;
       for (const auto& k : sb.classes)
         if (ce == cudaSuccess) ce = vqe::sweep_forward(k, nullptr, w, theta, ld_theta, with_grad, ctl, stream);
-      if (ce == cudaSuccess) ce = vqe::tc_hpsi(sb.tcb, nullptr, w, false, stream);
+      if (ce == cudaSuccess) ce = vqe::tc_hpsi(sb.tcb, nullptr, w, false, tctl, stream);
       if (ce == cudaSuccess) ce = vqe::sweep_dots(sb.d_sweep, nullptr, n, w, stream);
       if (with_grad)
         for (const auto& k : sb.classes)
@@ -3521,7 +3533,9 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
         ce = vqe::sweep_final(sb.d_sweep, nullptr, n, w, theta, ld_theta, ctl, energies, with_grad ? grads : nullptr,
                               ld_grad, stream);
       if (ce != cudaSuccess) return cuda_fail(ce, "batched cluster sweeps launch");
+      if ((rc = finish_slots())) return rc;
     } else {
+      if ((rc = finish_slots())) return rc;
       for (size_t k = 0; k < sb.mid.size(); ++k) {
         const size_t off = sb.mid_off[k];
         rc = run_one_by_one(b, std::vector<int>(1, sb.mid[k]), true, theta, ld_theta, energies, grads, ld_grad,
@@ -3699,7 +3713,8 @@ int vqe_batch_get_tuning(vqe_batch_t b, int* ctas_per_sm, int* gate_chunk, int* 
   if (ctas_per_sm) *ctas_per_sm = b->sb.ctas_per_sm;
   if (gate_chunk) *gate_chunk = b->sb.gate_chunk;
   if (grid) *grid = b->sb.slots.empty() ? b->sb.mid_ctas : b->sb.grid;
-  if (n_tasks) *n_tasks = (b->sb.q[1] ? int64_t(b->sb.q[1]->tasks.size()) : 0) + 2 * int64_t(b->sb.mid.size());
+  const int64_t mid = int64_t(b->sb.mid.size());  // two sweeps each, and one H psi
+  if (n_tasks) *n_tasks = (b->sb.q[1] ? int64_t(b->sb.q[1]->tasks.size()) : 0) + (mid ? 2 * mid + 1 : 0);
   return VQE_OK;
 }
 
@@ -3728,8 +3743,11 @@ int vqe_batch_status(vqe_batch_t b, const void* ws, size_t ws_bytes, vqe_stream_
   const int t = status - 1;
   const PersistQueue* Q = sb.q[sb.last_queue].get();
   std::string what = "task " + std::to_string(t);
-  if (Q && t >= 0 && size_t(t) < Q->tasks.size())
-    what += " (instance " + std::to_string(sb.descs[Q->tasks[t].slot].inst) + ")";
+  const int queued = Q ? int(Q->tasks.size()) : 0;
+  if (t < queued)
+    what += " (instance " + std::to_string(sb.descs[Q->tasks[size_t(t)].slot].inst) + ")";
+  else if (t == queued + 2 * int(sb.mid.size()))
+    what += " (H psi of the instances swept in cluster shared memory)";
   return fail(VQE_ERR_TIMEOUT, "persistent batch: a wait of " + what + " ran out of its " +
                                    std::to_string(sb.budget_ns) + " ns budget; outputs are NaN");
 }

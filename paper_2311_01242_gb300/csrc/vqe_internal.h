@@ -155,8 +155,16 @@ struct TcBatch {
 int tc_stages(int DbP, size_t smem_limit);
 int tc_tiles(const TcPlan& tc);
 cudaError_t tc_set_smem_limit(size_t bytes);
+// A batch's status word, what a wait that ran out writes there if nothing else did, and the
+// wait check (vqe_batch_set_wait). Single calls: none; their outputs are NaN.
+struct TcCtl {
+  int* status = nullptr;
+  int code = 0;
+  bool probe = false;
+  long long budget_ns = 0;
+};
 // lam_am (+)= the tensor-core part of H psi_am, for *one or every instance of B
-cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, cudaStream_t stream);
+cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, const TcCtl& ctl, cudaStream_t stream);
 inline TcBatch tc_single(const TcPlan& tc) {
   TcBatch b;
   b.n_tiles = tc_tiles(tc);
@@ -253,12 +261,12 @@ struct PersistDev {
   int32_t pad;
 };
 
-// memset of the counters, the persistent launch (grid CTAs), and the finalising
-// launch over rows[0, n_rows) (gradient rows first: n_grad_rows of them, skipped
-// when grad is null).
-cudaError_t batch_persistent_run(const PersistDev& p, int grid, size_t smem, const PFinal* rows, int n_rows,
-                                 int n_grad_rows, const double* theta, int64_t ld_theta, double* energy, double* grad,
-                                 int64_t ld_grad, cudaStream_t stream);
+// the persistent launch (grid CTAs; the counters are 0), and the finalising launch over
+// rows[0, n_rows) (gradient rows first: n_grad_rows of them, skipped when grad is null)
+cudaError_t batch_persistent_run(const PersistDev& p, int grid, size_t smem, const double* theta, int64_t ld_theta,
+                                 cudaStream_t stream);
+cudaError_t batch_persistent_final(const PersistDev& p, const PFinal* rows, int n_rows, int n_grad_rows,
+                                   double* energy, double* grad, int64_t ld_grad, cudaStream_t stream);
 cudaError_t set_persist_smem_limit(size_t smem);
 cudaError_t persist_occupancy(size_t smem, int* blocks_per_sm);
 // memset of the counters and the persistent launch alone (the gate sweeps of a
@@ -472,7 +480,7 @@ struct SweepCtl {                    // a batch's wait check (single calls: stat
   int* status;
   const int* never;
   long long budget_ns;
-  int probe, task0, n;               // forward sweeps are tasks task0 + i, reverse ones task0 + n + i
+  int probe, task0, n;               // forward sweeps are tasks task0 + i, reverse ones task0 + n + i, H psi task0 + 2 n
 };
 size_t sweep_smem(int M, int c, int shift, int64_t D, int threads);
 cudaError_t sweep_set_limits(size_t optin);

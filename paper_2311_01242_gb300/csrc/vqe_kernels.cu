@@ -922,7 +922,7 @@ cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuf
     if constexpr (REAL) {
       if (tc) {
         const TcInst one{sp.tc, b.tc, sp.str.ka, sp.str.kb, d.vals};
-        const cudaError_t e = tc_hpsi(tc_single(sp.tc), &one, b.base, sp.has_rest, stream);
+        const cudaError_t e = tc_hpsi(tc_single(sp.tc), &one, b.base, sp.has_rest, TcCtl{}, stream);
         if (e != cudaSuccess) return e;
       }
     }

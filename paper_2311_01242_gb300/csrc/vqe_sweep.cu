@@ -107,7 +107,7 @@ __device__ __forceinline__ unsigned long long clock_ns() {
 
 // The batch's wait check (vqe_batch_set_wait): the probed task waits for a count
 // that nothing reaches, for at most the budget, then records itself in the status
-// word; the outputs of every instance become NaN.
+// word; the outputs of every instance swept here or in the persistent launch become NaN.
 __device__ __forceinline__ void probe_wait(const SweepCtl& ctl, int task) {
   if (task != ctl.probe || threadIdx.x != 0) return;
   const unsigned long long t0 = clock_ns();

@@ -72,14 +72,15 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 // Waits for a barrier's phase for at most two seconds; then, or once another wait
 // of the block ran out, marks the block dead and returns (its row becomes NaN).
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* dead) {
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* dead,
+                                          unsigned long long budget_ns = 2000000000ull) {
   if (mbar_try(bar, parity)) return;
   const unsigned long long t0 = now_ns();
   for (int it = 0; it < (1 << 28); ++it) {
     if (mbar_try(bar, parity)) return;
     if ((it & 255) == 255) {
       if (*dead) return;
-      if (now_ns() - t0 > 2000000000ull) break;
+      if (now_ns() - t0 > budget_ns) break;
     }
   }
   *dead = 1;
@@ -360,7 +361,7 @@ struct TcShared {          // after the operand buffers and the lambda row
 // code.
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int2* __restrict__ work, int n_work,
-          int stages, int lam_len) {
+          int stages, int lam_len, const TcCtl ctl) {
   extern __shared__ __align__(1024) unsigned char raw[];
   unsigned char* base = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   unsigned char* sA = base;
@@ -392,6 +393,10 @@ k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = S.tmem;
+  if (ctl.probe && blockIdx.x == 0) {  // the wait check: a barrier that nothing reaches before the block's end
+    if (tid == 0) mbar_wait(smem_u32(&S.last), 0, &S.dead, static_cast<unsigned long long>(ctl.budget_ns));
+    __syncthreads();
+  }
 
   // pipeline positions, kept across rows and passes
   int st = 0;
@@ -596,6 +601,7 @@ k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int
     if (lane == 0) {  // nothing of this block is in flight when its tensor memory is given back
       tc_commit(smem_u32(&S.last));
       mbar_wait(smem_u32(&S.last), 0, &S.dead);
+      if (S.dead && ctl.status) atomicCAS(ctl.status, 0, ctl.code);
     }
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
@@ -746,7 +752,7 @@ struct GemmShared {
 
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_tc_onespin_gemm(const TcInst* __restrict__ many, const TcInst one, char* ws, const int2* __restrict__ work,
-                  int n_work, int add) {
+                  int n_work, int add, const TcCtl ctl) {
   extern __shared__ __align__(1024) unsigned char raw[];
   unsigned char* ring = raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u);
   GemmShared& S = *reinterpret_cast<GemmShared*>(ring + kRing * kPairBytes);
@@ -952,6 +958,7 @@ k_tc_onespin_gemm(const TcInst* __restrict__ many, const TcInst one, char* ws, c
     if (lane == 0) {
       tc_commit(smem_u32(&S.last));
       mbar_wait(smem_u32(&S.last), 0, &S.dead);
+      if (S.dead && ctl.status) atomicCAS(ctl.status, 0, ctl.code);
     }
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
@@ -982,7 +989,7 @@ cudaError_t tc_set_smem_limit(size_t bytes) {
 
 int tc_tiles(const TcPlan& tc) { return (tc.Da + kRows - 1) / kRows * (tc.DbP / kTileN); }
 
-cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, cudaStream_t stream) {
+cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, const TcCtl& ctl, cudaStream_t stream) {
   const TcInst none{};
   const TcInst& o = one ? *one : none;
   const TcInst* many = one ? nullptr : B.insts;
@@ -992,8 +999,9 @@ cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, cud
   k_tc_onespin<<<dim3(unsigned(B.Da), n), 256, size_t(B.DaP) * 8, stream>>>(many, o, ws, 0);
   k_tc_onespin<<<dim3(unsigned(B.Db), n), 256, size_t(B.DbP) * 8, stream>>>(many, o, ws, 1);
   const int tg = B.n_tiles < B.sms ? B.n_tiles : B.sms, rg = B.n_rows < B.sms ? B.n_rows : B.sms;
-  k_tc_onespin_gemm<<<tg, kGemmThreads, gemm_smem(), stream>>>(many, o, ws, B.tiles, B.n_tiles, add ? 1 : 0);
-  k_tc_hops<<<rg, kThreads, hops_smem(B.DbP, B.stages), stream>>>(many, o, ws, B.rows, B.n_rows, B.stages, B.DbP);
+  k_tc_onespin_gemm<<<tg, kGemmThreads, gemm_smem(), stream>>>(many, o, ws, B.tiles, B.n_tiles, add ? 1 : 0, ctl);
+  k_tc_hops<<<rg, kThreads, hops_smem(B.DbP, B.stages), stream>>>(many, o, ws, B.rows, B.n_rows, B.stages, B.DbP,
+                                                                 ctl);
   return cudaGetLastError();
 }
 
