@@ -82,8 +82,11 @@ int vqe_version(void);
  *                            a cluster of two;
  *   VQE_FLAG_FP64_SWEEPS     run the gate sweeps in FP64 instead of 64-bit fixed
  *                            point: in the resident kernel, and with a launch
- *                            per gate (or VQE_FLAG_PERSISTENT_SWEEPS) where they
- *                            run in cluster shared memory or by groups of gates;
+ *                            per gate (or VQE_FLAG_PERSISTENT_SWEEPS; in batches
+ *                            the persistent launch) where they run in cluster
+ *                            shared memory or by groups of gates. A batch has a
+ *                            plan of its own for this flag, built by the first
+ *                            vqe_batch_workspace_bytes or call under it;
  *   VQE_FLAG_NO_STRINGS      streaming H psi by connectivity rows (or a scan of
  *                            all groups) instead of alpha/beta strings;
  *   VQE_FLAG_PERSISTENT_SWEEPS streaming gate sweeps of a single instance as
@@ -351,17 +354,24 @@ int vqe_pool_gradients(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_ansatz_t pool,
  * A batch of independent instances (the paper runs hundreds of independent
  * simulation jobs over geometries and molecules, abstract and Sec. 4).
  * Instances whose sector and tables fit shared memory run in one resident
- * launch (a CTA pair each). All other instances run in ONE persistent launch:
- * a device work queue of tasks (per instance: HF init, each gate's rotation on
- * a range of pairs, H psi on a range of output strings or rows, the energy's
- * partial sums, each gate's adjoint step and gradient partials), taken in a
- * fixed list-scheduled order by a grid sized to the device, where a task waits
- * (bounded in time, see vqe_batch_set_wait) only for the earlier tasks of its
- * own instance; a small finalising launch then sums the partials. Instances
- * with a gate or sector of more than 262,144 pairs or states are evaluated
- * after it, one by one. Results equal vqe_energy_grad's on each instance bit
- * for bit. hams/ansatze: n_inst handles (they may repeat) that must outlive
- * the batch. Synchronous; allocates the batch's device descriptors and queues.
+ * launch (a CTA pair each). Of the others,
+ *   - spin sectors of 256 to 131,072 states whose H psi is wholly on the tensor
+ *     cores (every Jordan-Wigner Hamiltonian) sweep their gates in cluster
+ *     shared memory, all in a few launches side by side, around one launch
+ *     sequence of H psi for all of them;
+ *   - sectors of at most 262,144 states without that H psi (boson and other
+ *     electron-number sectors, Hamiltonians of other forms) run in ONE
+ *     persistent launch: a device work queue of tasks (per instance: HF init,
+ *     each gate's rotation on a range of pairs, H psi on a range of output
+ *     strings or rows, the energy's partial sums, each gate's adjoint step and
+ *     gradient partials), taken in a fixed list-scheduled order by a grid sized
+ *     to the device, where a task waits (bounded in time, see
+ *     vqe_batch_set_wait) only for the earlier tasks of its own instance; a
+ *     small finalising launch then sums the partials;
+ *   - the rest are evaluated after them, one by one.
+ * Results equal vqe_energy_grad's on each instance bit for bit. hams/ansatze:
+ * n_inst handles (they may repeat) that must outlive the batch. Synchronous;
+ * allocates the batch's device descriptors and queues.
  */
 int vqe_create_batch(int n_inst, const vqe_hamiltonian_t* hams,
                      const vqe_ansatz_t* ansatze, vqe_batch_t* out);

@@ -96,7 +96,7 @@ k_batch_persistent(const PersistDev p, const double* __restrict__ theta, int64_t
   int* status = p.counters + p.n + 1;
   for (;;) {
     if (tid == 0) {
-      int t = ld_acquire(status) != 0 ? INT_MAX : atomicAdd(next, 1);
+      int t = ld_acquire(status) != 0 ? INT_MAX : p.first + atomicAdd(next, 1);
       int ok = 0;
       if (t < p.n_tasks) {
         const PTask& tk = p.tasks[t];

@@ -389,6 +389,7 @@ struct vqe_ansatz_s {
 // tuning changes.
 struct PersistQueue {
   std::vector<vqe::PTask> tasks;  // queue order
+  int32_t split = 0;              // tasks before the H psi of the slots that run it on the tensor cores
   std::vector<vqe::PFinal> finals;
   int n_grad_rows = 0;
   vqe::PTask* d_tasks = nullptr;
@@ -400,7 +401,9 @@ struct PersistQueue {
 };
 
 struct StreamBatch {
+  bool fp64 = false;                      // the plan for VQE_FLAG_FP64_SWEEPS: no cluster sweeps
   std::vector<int> slots;                 // batch index of each persistent slot
+  std::vector<char> slot_tc;              // with fp64: their H psi is tcb's, between two launches
   std::vector<int> big;                   // batch indices evaluated one by one (too large for a slot)
   std::vector<int> mid;                   // batch indices swept in cluster shared memory
   std::vector<size_t> mid_off;            // their workspace layouts
@@ -423,7 +426,6 @@ struct StreamBatch {
   int gate_chunk = 1024;                  // pairs per FWD/ADJ task (multiple of 256)
   long long budget_ns = 2000000000ll;
   int probe_task = -1;
-  int last_queue = 1;                     // queue of the last launch (for status messages)
   ~StreamBatch() {
     dfree(d_sweep);
     dfree(d_tc);
@@ -459,6 +461,10 @@ struct vqe_batch_s {
   int n_inst = 0;
   int32_t max_params = 0;
   StreamBatch sb;
+  std::unique_ptr<StreamBatch> sb64;    // under VQE_FLAG_FP64_SWEEPS, built on first use
+  std::mutex sb64_mu;
+  std::atomic<const StreamBatch*> last{nullptr};  // of the last launch (for the status word),
+  std::atomic<int> last_queue{1};                 // and its queue (for the message)
   HostGraph hg;
   uint64_t tuning_version = 0;
   cudaStream_t capture_stream = nullptr;  // private stream the host-call graph is captured on
@@ -1533,7 +1539,8 @@ bool resident_fit(vqe_ansatz_t a, const vqe_hamiltonian_s::Ell* e, bool real, In
 struct WsLayout {
   size_t psi, lam, psi_am, lam_am, cs, epart, ctr, gpart, phi, total;
   bool has_tc;
-  vqe::TcOffsets tc;  // tensor-core H psi
+  vqe::TcOffsets tc;  // tensor-core H psi, from tc.dig to tc_end
+  size_t tc_end;
   size_t sw_phi, sw_gacc, sw_dot;  // sweeps in cluster shared memory
   size_t gr_trig, gr_gacc, gr_norm;  // sweeps by groups of gates
 };
@@ -1619,6 +1626,7 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
     L.tc.psi_am = int64_t(L.psi_am);
     L.tc.lam_am = int64_t(L.lam_am);
   }
+  L.tc_end = L.total;
   L.sw_phi = L.sw_gacc = L.sw_dot = 0;
   if (L.has_tc && mid_ansatz(a)) {
     L.sw_gacc = L.total;
@@ -2993,8 +3001,9 @@ int vqe_pool_gradients(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_ansatz_t pool, c
 // schedule of rough task costs over the grid's CTAs: whenever a CTA frees up,
 // it takes the ready task whose level has the longest remaining chain after it
 // (critical path first), so long instances start early and short ones fill in.
-static int build_queues(vqe_batch_s* B) {
-  StreamBatch& sb = B->sb;
+// Slots whose H psi runs on the tensor cores (slot_tc) have no such task: the queue is
+// split into what comes before it and what comes after, two launches.
+static int build_queues(vqe_batch_s* B, StreamBatch& sb) {
   const int n = int(sb.slots.size());
   const int64_t gc = sb.gate_chunk;
   for (int mode = 0; mode < 2; ++mode) {
@@ -3003,6 +3012,7 @@ static int build_queues(vqe_batch_s* B) {
       int slot;
       int64_t t0, nt;  // first task (in `tasks`) and count
       double cost, bottom;
+      bool late;       // after the split
     };
     std::vector<vqe::PTask> tasks;
     std::vector<double> cost;
@@ -3017,11 +3027,12 @@ static int build_queues(vqe_batch_s* B) {
       int rc2 = VQE_OK;
       const auto* e = get_ell(B->hams[bi], a, &rc2);
       if (!e) return rc2;
-      const bool str = d.str != nullptr;
+      const bool str = d.str != nullptr, tc = sb.fp64 && sb.slot_tc[size_t(s)];
+      bool late = false;
       int32_t done = 0;  // tasks of the slot in earlier levels
       slot_lv0[s] = int64_t(lv.size());
       auto level = [&](auto&& add) {
-        Lvl L{s, int64_t(tasks.size()), 0, 0.0, 0.0};
+        Lvl L{s, int64_t(tasks.size()), 0, 0.0, 0.0, late};
         add();
         L.nt = int64_t(tasks.size()) - L.t0;
         if (L.nt == 0) return;
@@ -3059,7 +3070,7 @@ static int build_queues(vqe_batch_s* B) {
         level([&] {
           for (int64_t lo = 0; lo < D; lo += ch) task(vqe::PT_GATHER, 0, lo, std::min(D, lo + ch), 0, 1500.0 + 0.3 * double(std::min(ch, D - lo)));
         });
-      level([&] {
+      if (!tc) level([&] {
         const double per_entry = 1.6;  // measured order of magnitude of the string-driven H psi per CTA
         if (str) {
           const int Da = e->str.Da, Db = e->str.Db;
@@ -3075,6 +3086,7 @@ static int build_queues(vqe_batch_s* B) {
           }
         }
       });
+      late = true;
       if (str)
         level([&] {
           for (int64_t lo = 0; lo < D; lo += ch) task(vqe::PT_SCATTER, 0, lo, std::min(D, lo + ch), 0, 1500.0 + 0.3 * double(std::min(ch, D - lo)));
@@ -3118,7 +3130,14 @@ static int build_queues(vqe_batch_s* B) {
     std::priority_queue<PQ, std::vector<PQ>, std::greater<PQ>> running;
     std::vector<int64_t> left(lv.size());
     for (int64_t l = 0; l < int64_t(lv.size()); ++l) left[l] = lv[l].nt;
+    const bool split = std::find(sb.slot_tc.begin(), sb.slot_tc.end(), char(1)) != sb.slot_tc.end();
+    bool after = !split;  // levels after the split are ready too
+    std::vector<int64_t> held;
     auto push_level = [&](int64_t l) {
+      if (!after && lv[l].late) {
+        held.push_back(l);
+        return;
+      }
       for (int64_t t = lv[l].t0; t < lv[l].t0 + lv[l].nt; ++t) ready.push(std::make_pair(lv[l].bottom, -t));
     };
     for (int s = 0; s < n; ++s)
@@ -3127,6 +3146,11 @@ static int build_queues(vqe_batch_s* B) {
     double now = 0.0;
     Q->tasks.reserve(tasks.size());
     while (Q->tasks.size() < tasks.size()) {
+      if (!after && running.empty() && ready.empty()) {
+        after = true;
+        Q->split = int32_t(Q->tasks.size());
+        for (int64_t l : held) push_level(l);
+      }
       while (free_ctas > 0 && !ready.empty()) {
         const int64_t t = -ready.top().second;
         ready.pop();
@@ -3204,11 +3228,45 @@ static int persist_grid(const StreamBatch& sb, int* grid) {
   return VQE_OK;
 }
 
+// The tensor-core H psi of many instances: the largest sizes and the work lists (costly
+// instances first).
+static int build_tc_lists(StreamBatch& sb, const std::vector<vqe::TcInst>& tcs) {
+  size_t optin = 0;
+  int sms = 0, rc;
+  if ((rc = device_limits(&optin, &sms))) return rc;
+  std::vector<std::pair<int64_t, int>> order;
+  vqe::TcBatch& t = sb.tcb;
+  for (size_t i = 0; i < tcs.size(); ++i) {
+    const vqe::TcPlan& T = tcs[i].tc;
+    order.push_back({-int64_t(T.DbP) * T.K, int(i)});
+    t.items = std::max(t.items, int(T.items));
+    t.Da = std::max(t.Da, int(T.Da));
+    t.Db = std::max(t.Db, int(T.Db));
+    t.DaP = std::max(t.DaP, int(T.DaP));
+    t.DbP = std::max(t.DbP, int(T.DbP));
+    t.stages = i ? std::min(t.stages, int(T.stages)) : int(T.stages);
+  }
+  std::sort(order.begin(), order.end());
+  std::vector<int2> tiles, rows;
+  for (const auto& o : order) {
+    const vqe::TcPlan& T = tcs[size_t(o.second)].tc;
+    for (int k = 0; k < vqe::tc_tiles(T); ++k) tiles.push_back(make_int2(o.second, k));
+    for (int r = 0; r < T.Da; ++r) rows.push_back(make_int2(o.second, r));
+  }
+  if ((rc = upload(tcs, &sb.d_tc)) || (rc = upload(tiles, &sb.d_tiles)) || (rc = upload(rows, &sb.d_rows))) return rc;
+  t.insts = sb.d_tc;
+  t.tiles = sb.d_tiles;
+  t.rows = sb.d_rows;
+  t.n = int(tcs.size());
+  t.n_tiles = int(tiles.size());
+  t.n_rows = int(rows.size());
+  t.sms = sms;
+  return VQE_OK;
+}
+
 // The batch's instances swept in cluster shared memory: workspace layouts after the
-// persistent slots', cluster sizes, and the tensor-core work lists (costly instances
-// first).
-static int build_mid_batch(vqe_batch_s* B) {
-  StreamBatch& sb = B->sb;
+// persistent slots' and cluster sizes.
+static int build_mid_batch(vqe_batch_s* B, StreamBatch& sb) {
   const int n = int(sb.mid.size());
   if (n == 0) return VQE_OK;
   size_t optin = 0;
@@ -3247,7 +3305,6 @@ static int build_mid_batch(vqe_batch_s* B) {
   sb.mid_ctas = total;
   std::vector<vqe::SweepInst> sweep;
   std::vector<vqe::TcInst> tcs;
-  std::vector<std::pair<int64_t, int>> order;
   size_t off = sb.persist_bytes;
   std::vector<size_t> first;
   for (int i = 0; i < n; ++i) {
@@ -3257,15 +3314,6 @@ static int build_mid_batch(vqe_batch_s* B) {
     const WsLayout L = ws_layout(B->ans[b], false, true);
     sb.mid_off.push_back(off);
     tcs.push_back(tc_inst(B->hams[b], e, L, off));
-    order.push_back({-int64_t(e->tc.DbP) * e->tc.K, i});
-    const vqe::TcPlan& T = e->tc;
-    vqe::TcBatch& t = sb.tcb;
-    t.items = std::max(t.items, int(T.items));
-    t.Da = std::max(t.Da, int(T.Da));
-    t.Db = std::max(t.Db, int(T.Db));
-    t.DaP = std::max(t.DaP, int(T.DaP));
-    t.DbP = std::max(t.DbP, int(T.DbP));
-    t.stages = i ? std::min(t.stages, int(T.stages)) : int(T.stages);
     off += L.total;
   }
   for (int c = 16; c >= 1; c /= 2) {
@@ -3296,44 +3344,29 @@ static int build_mid_batch(vqe_batch_s* B) {
     else
       first.pop_back();
   }
-  std::sort(order.begin(), order.end());
-  std::vector<int2> tiles, rows;
-  for (const auto& o : order) {
-    const vqe::TcPlan& T = tcs[size_t(o.second)].tc;
-    for (int t = 0; t < vqe::tc_tiles(T); ++t) tiles.push_back(make_int2(o.second, t));
-    for (int r = 0; r < T.Da; ++r) rows.push_back(make_int2(o.second, r));
-  }
-  if ((rc = upload(sweep, &sb.d_sweep)) || (rc = upload(tcs, &sb.d_tc)) || (rc = upload(tiles, &sb.d_tiles)) ||
-      (rc = upload(rows, &sb.d_rows)))
-    return rc;
+  if ((rc = upload(sweep, &sb.d_sweep)) || (rc = build_tc_lists(sb, tcs))) return rc;
   for (size_t k = 0; k < sb.classes.size(); ++k) sb.classes[k].insts = sb.d_sweep + first[k];
-  vqe::TcBatch& t = sb.tcb;
-  t.insts = sb.d_tc;
-  t.tiles = sb.d_tiles;
-  t.rows = sb.d_rows;
-  t.n = n;
-  t.n_tiles = int(tiles.size());
-  t.n_rows = int(rows.size());
-  t.sms = sms;
   sb.persist_bytes = off;
   return VQE_OK;
 }
 
-static int build_stream_batch(vqe_batch_s* B) {
-  StreamBatch& sb = B->sb;
+static int build_stream_batch(vqe_batch_s* B, StreamBatch& sb) {
   for (int i : B->streaming[0]) {
     int rc = VQE_OK;
     const auto* e = get_ell(B->hams[i], B->ans[i], &rc);
     if (!e) return rc;
-    if (mid_fits(B->ans[i], e))
+    if (!sb.fp64 && mid_fits(B->ans[i], e)) {
       sb.mid.push_back(i);
-    else if (slot_fits(B->ans[i]) && !e->use_tc)
+    } else if (slot_fits(B->ans[i]) && (sb.fp64 || !e->use_tc)) {
       sb.slots.push_back(i);
-    else
+      sb.slot_tc.push_back(e->use_tc ? 1 : 0);
+    } else {
       sb.big.push_back(i);
+    }
   }
-  for (int i : sb.big)
-    if (group_ansatz(B->ans[i])) get_groups(B->ans[i], nullptr);
+  if (!sb.fp64)
+    for (int i : sb.big)
+      if (group_ansatz(B->ans[i])) get_groups(B->ans[i], nullptr);
   for (int i : sb.big) sb.big_bytes = std::max(sb.big_bytes, ws_layout(B->ans[i], false, true).total);
   const int n = int(sb.slots.size());
   if (n == 0 && sb.mid.empty()) return VQE_OK;
@@ -3373,12 +3406,61 @@ static int build_stream_batch(vqe_batch_s* B) {
   sb.counters_off = off;
   sb.persist_bytes = off + align256(size_t(n + 3) * sizeof(int));  // and one that stays zero
   int rc;
-  if ((rc = build_mid_batch(B))) return rc;
+  if ((rc = build_mid_batch(B, sb))) return rc;
   if (n == 0) return VQE_OK;
+  std::vector<vqe::TcInst> tcs;
+  for (int s = 0; s < n; ++s) {
+    if (!sb.slot_tc[size_t(s)]) continue;
+    const int i = sb.slots[s];
+    const auto* e = get_ell(B->hams[i], B->ans[i], &rc);
+    if (!e) return rc;
+    const WsLayout L = ws_layout(B->ans[i], false, false);
+    vqe::TcInst t = tc_inst(B->hams[i], e, L, sb.persist_bytes - size_t(L.tc.dig));
+    t.off.psi_am = sb.pslots[size_t(s)].psi_am;
+    t.off.lam_am = sb.pslots[size_t(s)].lam_am;
+    tcs.push_back(t);
+    sb.persist_bytes += L.tc_end - size_t(L.tc.dig);
+  }
+  if (!tcs.empty() && (rc = build_tc_lists(sb, tcs))) return rc;
   if ((rc = upload(sb.descs, &sb.d_desc))) return rc;
   if ((rc = upload(sb.pslots, &sb.d_slots))) return rc;
   if ((rc = persist_grid(sb, &sb.grid))) return rc;
-  return build_queues(B);
+  return build_queues(B, sb);
+}
+
+// The plan of the batch's streamed real instances under the flags: VQE_FLAG_FP64_SWEEPS
+// has one of its own, where all that fit a slot sweep in the persistent launch (in front
+// of and after one launch sequence of H psi on the tensor cores): by launches per gate,
+// one instance after the other, 12 instances of 14 to 18 qubits took 5.5 ms, 2.6 before
+// there were cluster sweeps. Built on first use, or null if that is inside a stream capture.
+static StreamBatch* fp64_batch(vqe_batch_t b, cudaStream_t stream) {
+  std::lock_guard<std::mutex> lk(b->sb64_mu);
+  if (b->sb64) return b->sb64.get();
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  std::unique_ptr<StreamBatch> p(new StreamBatch);
+  p->fp64 = true;
+  p->ctas_per_sm = b->sb.ctas_per_sm;
+  p->gate_chunk = b->sb.gate_chunk;
+  p->budget_ns = b->sb.budget_ns;
+  p->probe_task = b->sb.probe_task;
+  if (build_stream_batch(b, *p) != VQE_OK) return nullptr;
+  b->sb64 = std::move(p);
+  return b->sb64.get();
+}
+static bool fp64_differs(vqe_batch_t b) {
+  if ((g_flags & VQE_FLAG_FP64_SWEEPS) == 0) return false;
+  if (!b->sb.mid.empty()) return true;
+  for (int i : b->sb.big)
+    if (slot_fits(b->ans[i])) return true;
+  return false;
+}
+static StreamBatch* stream_batch(vqe_batch_t b, cudaStream_t stream) {
+  StreamBatch* p = fp64_differs(b) ? fp64_batch(b, stream) : nullptr;
+  return p ? p : &b->sb;
 }
 
 int vqe_create_batch(int n_inst, const vqe_hamiltonian_t* hams, const vqe_ansatz_t* ans, vqe_batch_t* out) {
@@ -3413,7 +3495,7 @@ int vqe_create_batch(int n_inst, const vqe_hamiltonian_t* hams, const vqe_ansatz
     int rc = upload(B->res_descs[mode], &B->d_res[mode]);
     if (rc) return rc;
   }
-  int rc = build_stream_batch(B.get());
+  int rc = build_stream_batch(B.get(), B->sb);
   if (rc) return rc;
   *out = B.release();
   return VQE_OK;
@@ -3423,20 +3505,29 @@ int32_t vqe_batch_max_params(vqe_batch_t b) { return b ? b->max_params : 0; }
 
 // Streamed instances run one by one (stream_energy_grad) in complex mode, under
 // VQE_FLAG_NO_STRINGS, and for instances too large for a persistent slot.
-static bool persistent_mode(vqe_batch_t b, bool real) {
-  return real && !(g_flags & VQE_FLAG_NO_STRINGS) && !(b->sb.slots.empty() && b->sb.mid.empty());
+static bool persistent_mode(const StreamBatch& sb, bool real) {
+  return real && !(g_flags & VQE_FLAG_NO_STRINGS) && !(sb.slots.empty() && sb.mid.empty());
+}
+
+static size_t batch_need(vqe_batch_t b, const StreamBatch& sb, bool with_grad) {
+  const int mode = use_real() ? 0 : 1;
+  size_t one = 0;  // largest one-by-one instance
+  if (persistent_mode(sb, mode == 0)) {
+    for (int i : sb.big) one = std::max(one, ws_layout(b->ans[i], false, with_grad).total);
+    return sb.persist_bytes + one;
+  }
+  for (int i : b->streaming[mode]) one = std::max(one, ws_layout(b->ans[i], mode == 1, with_grad).total);
+  return one;
+}
+
+// a workspace sized under other flags is enough if it holds the plan without them
+static const StreamBatch* batch_plan(vqe_batch_t b, bool with_grad, size_t ws_bytes, cudaStream_t stream) {
+  const StreamBatch* p = stream_batch(b, stream);
+  return ws_bytes < batch_need(b, *p, with_grad) ? &b->sb : p;
 }
 
 size_t vqe_batch_workspace_bytes(vqe_batch_t b, int with_grad) {
-  if (!b) return 0;
-  const int mode = use_real() ? 0 : 1;
-  size_t one = 0;  // largest one-by-one instance
-  if (mode == 0 && persistent_mode(b, true)) {
-    for (int i : b->sb.big) one = std::max(one, ws_layout(b->ans[i], false, with_grad != 0).total);
-    return b->sb.persist_bytes + one;
-  }
-  for (int i : b->streaming[mode]) one = std::max(one, ws_layout(b->ans[i], mode == 1, with_grad != 0).total);
-  return one;
+  return b ? batch_need(b, *stream_batch(b, nullptr), with_grad != 0) : 0;
 }
 
 static int run_one_by_one(vqe_batch_t b, const std::vector<int>& which, bool real, const double* theta,
@@ -3477,11 +3568,11 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
                                           use_fixed(real));
     if (ce != cudaSuccess) return cuda_fail(ce, "batched resident launch");
   }
-  if (persistent_mode(b, real)) {
-    const StreamBatch& sb = b->sb;
-    const size_t need = vqe_batch_workspace_bytes(b, with_grad);
-    if ((rc = check_ws(ws, ws_bytes, need))) return rc;
-    b->sb.last_queue = with_grad ? 1 : 0;
+  const StreamBatch& sb = *batch_plan(b, with_grad, ws_bytes, stream);
+  if (persistent_mode(sb, real)) {
+    if ((rc = check_ws(ws, ws_bytes, batch_need(b, sb, with_grad)))) return rc;
+    b->last = &sb;
+    b->last_queue = with_grad ? 1 : 0;
     int* counters = reinterpret_cast<int*>(static_cast<char*>(ws) + sb.counters_off);
     const int n_slots = int(sb.slots.size());
     int queued = 0;
@@ -3493,15 +3584,28 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
       pd.desc = sb.d_desc;
       pd.slots = sb.d_slots;
       pd.tasks = Q.d_tasks;
-      pd.n_tasks = queued = int32_t(Q.tasks.size());
+      queued = int32_t(Q.tasks.size());
+      pd.n_tasks = Q.split ? Q.split : queued;
       pd.n = int32_t(n_slots);
       pd.ws = static_cast<char*>(ws);
       pd.counters = counters;
       pd.budget_ns = sb.budget_ns;
       pd.probe_task = sb.probe_task;
-      pd.pad = 0;
+      pd.first = 0;
       if ((rc = ensure_persist_smem(sb.smem))) return rc;
       ce = vqe::batch_persistent_run(pd, sb.grid, sb.smem, theta, ld_theta, stream);
+      if (ce == cudaSuccess && Q.split) {
+        vqe::TcCtl tctl;
+        tctl.status = counters + n_slots + 1;
+        tctl.code = queued + 1;
+        tctl.probe = sb.probe_task == queued;
+        tctl.budget_ns = sb.budget_ns;
+        ce = vqe::tc_hpsi(sb.tcb, nullptr, pd.ws, false, tctl, stream);
+        if (ce == cudaSuccess) ce = cudaMemsetAsync(counters + n_slots, 0, sizeof(int), stream);
+        pd.first = Q.split;
+        pd.n_tasks = queued;
+        if (ce == cudaSuccess) ce = vqe::batch_persistent_run(pd, sb.grid, sb.smem, theta, ld_theta, stream);
+      }
       if (ce != cudaSuccess) return cuda_fail(ce, "persistent batch launch");
     }
     // outputs last: a wait of either kind that runs out makes all of them NaN
@@ -3547,8 +3651,7 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
       return run_one_by_one(b, sb.big, true, theta, ld_theta, energies, grads, ld_grad,
                             static_cast<char*>(ws) + sb.persist_bytes, ws_bytes - sb.persist_bytes, stream);
   } else if (!b->streaming[mode].empty()) {
-    const size_t need = vqe_batch_workspace_bytes(b, with_grad);
-    if ((rc = check_ws(ws, ws_bytes, need))) return rc;
+    if ((rc = check_ws(ws, ws_bytes, batch_need(b, sb, with_grad)))) return rc;
     return run_one_by_one(b, b->streaming[mode], real, theta, ld_theta, energies, grads, ld_grad,
                           static_cast<char*>(ws), ws_bytes, stream);
   }
@@ -3579,7 +3682,8 @@ int vqe_batch_energy_grad_host(vqe_batch_t b, const double* theta_host, int64_t 
   const int64_t Mx = std::max(b->max_params, 1);
   if (ld_theta < b->max_params || (with_grad && ld_grad < b->max_params))
     return fail(VQE_ERR_INVALID_ARG, "leading dimension smaller than max params");
-  const size_t need = vqe_batch_host_workspace_bytes(b, with_grad);
+  size_t need = vqe_batch_host_workspace_bytes(b, with_grad);
+  if (ws_bytes < need) need -= batch_need(b, *stream_batch(b, nullptr), with_grad) - batch_need(b, b->sb, with_grad);
   int rc = check_ws(ws, ws_bytes, need);
   if (rc) return rc;
   char* base = static_cast<char*>(ws);
@@ -3619,7 +3723,7 @@ int vqe_batch_energy_grad_host(vqe_batch_t b, const double* theta_host, int64_t 
   // after the synchronisation: a wait of the persistent launch that ran out
   // (status word in the batch's part of the workspace) returns VQE_ERR_TIMEOUT
   auto persist_check = [&]() -> int {
-    if (!persistent_mode(b, use_real())) return VQE_OK;
+    if (!persistent_mode(*batch_plan(b, with_grad, ws_bytes - off, stream), use_real())) return VQE_OK;
     return vqe_batch_status(b, base + off, ws_bytes - off, stream);
   };
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -3684,17 +3788,18 @@ int vqe_batch_set_tuning(vqe_batch_t b, int ctas_per_sm, int gate_chunk, int swe
   if (sweep_threads != 0 && (sweep_threads < 32 || sweep_threads > vqe::kResidentThreads || sweep_threads % 32))
     return fail(VQE_ERR_INVALID_ARG, "sweep_threads: a multiple of 32 in [32, 512], or 0 to keep");
   ++b->tuning_version;  // launch shapes are captured in the host-call graph
-  StreamBatch& sb = b->sb;
-  const bool changed = ctas_per_sm != sb.ctas_per_sm || (gate_chunk && gate_chunk != sb.gate_chunk);
-  if (changed && !(sb.slots.empty() && sb.mid.empty())) {
-    sb.ctas_per_sm = ctas_per_sm;
-    if (gate_chunk) sb.gate_chunk = gate_chunk;
-  }
-  if (changed && !sb.slots.empty()) {  // (cluster sweeps have no such choice)
-    int rc = persist_grid(sb, &sb.grid);
-    if (rc == VQE_OK) rc = build_queues(b);
+  std::unique_lock<std::mutex> lk(b->sb64_mu);
+  for (StreamBatch* sb : {&b->sb, b->sb64.get()}) {
+    if (!sb || (sb->slots.empty() && sb->mid.empty())) continue;
+    if (ctas_per_sm == sb->ctas_per_sm && (!gate_chunk || gate_chunk == sb->gate_chunk)) continue;
+    sb->ctas_per_sm = ctas_per_sm;
+    if (gate_chunk) sb->gate_chunk = gate_chunk;
+    if (sb->slots.empty()) continue;  // (cluster sweeps have no such choice)
+    int rc = persist_grid(*sb, &sb->grid);
+    if (rc == VQE_OK) rc = build_queues(b, *sb);
     if (rc) return rc;
   }
+  lk.unlock();
   if (sweep_threads) {
     for (int mode = 0; mode < 2; ++mode) {
       for (auto& d : b->res_descs[mode]) d.sweep_threads = sweep_threads;
@@ -3710,11 +3815,13 @@ int vqe_batch_set_tuning(vqe_batch_t b, int ctas_per_sm, int gate_chunk, int swe
 
 int vqe_batch_get_tuning(vqe_batch_t b, int* ctas_per_sm, int* gate_chunk, int* grid, int64_t* n_tasks) {
   if (!b) return fail(VQE_ERR_INVALID_ARG, "NULL batch");
-  if (ctas_per_sm) *ctas_per_sm = b->sb.ctas_per_sm;
-  if (gate_chunk) *gate_chunk = b->sb.gate_chunk;
-  if (grid) *grid = b->sb.slots.empty() ? b->sb.mid_ctas : b->sb.grid;
-  const int64_t mid = int64_t(b->sb.mid.size());  // two sweeps each, and one H psi
-  if (n_tasks) *n_tasks = (b->sb.q[1] ? int64_t(b->sb.q[1]->tasks.size()) : 0) + (mid ? 2 * mid + 1 : 0);
+  const StreamBatch& sb = *stream_batch(b, nullptr);
+  if (ctas_per_sm) *ctas_per_sm = sb.ctas_per_sm;
+  if (gate_chunk) *gate_chunk = sb.gate_chunk;
+  if (grid) *grid = sb.slots.empty() ? sb.mid_ctas : sb.grid;
+  // two sweeps for each instance in cluster shared memory, and one H psi on the tensor cores
+  if (n_tasks)
+    *n_tasks = (sb.q[1] ? int64_t(sb.q[1]->tasks.size()) : 0) + 2 * int64_t(sb.mid.size()) + (sb.tcb.n_rows ? 1 : 0);
   return VQE_OK;
 }
 
@@ -3724,14 +3831,19 @@ int vqe_batch_set_wait(vqe_batch_t b, int64_t budget_ns, int32_t probe_task) {
     return fail(VQE_ERR_INVALID_ARG, "budget_ns: 1e3 .. 6e11");
   if (probe_task < -1) return fail(VQE_ERR_INVALID_ARG, "probe_task: a task index, or -1");
   ++b->tuning_version;
-  b->sb.budget_ns = budget_ns;
-  b->sb.probe_task = probe_task;
+  std::lock_guard<std::mutex> lk(b->sb64_mu);
+  for (StreamBatch* sb : {&b->sb, b->sb64.get()})
+    if (sb) {
+      sb->budget_ns = budget_ns;
+      sb->probe_task = probe_task;
+    }
   return VQE_OK;
 }
 
 int vqe_batch_status(vqe_batch_t b, const void* ws, size_t ws_bytes, vqe_stream_t stream) {
   if (!b) return fail(VQE_ERR_INVALID_ARG, "NULL batch");
-  const StreamBatch& sb = b->sb;
+  const StreamBatch* last = b->last;
+  const StreamBatch& sb = last ? *last : b->sb;
   if (sb.slots.empty() && sb.mid.empty()) return VQE_OK;
   if (!ws || ws_bytes < sb.persist_bytes) return fail(VQE_ERR_WORKSPACE, "workspace smaller than the batch's");
   int status = 0;
@@ -3741,13 +3853,13 @@ int vqe_batch_status(vqe_batch_t b, const void* ws, size_t ws_bytes, vqe_stream_
   if (ce != cudaSuccess) return cuda_fail(ce, "status read");
   if (status == 0) return VQE_OK;
   const int t = status - 1;
-  const PersistQueue* Q = sb.q[sb.last_queue].get();
+  const PersistQueue* Q = sb.q[b->last_queue].get();
   std::string what = "task " + std::to_string(t);
   const int queued = Q ? int(Q->tasks.size()) : 0;
   if (t < queued)
     what += " (instance " + std::to_string(sb.descs[Q->tasks[size_t(t)].slot].inst) + ")";
   else if (t == queued + 2 * int(sb.mid.size()))
-    what += " (H psi of the instances swept in cluster shared memory)";
+    what += " (H psi on the tensor cores)";
   return fail(VQE_ERR_TIMEOUT, "persistent batch: a wait of " + what + " ran out of its " +
                                    std::to_string(sb.budget_ns) + " ns budget; outputs are NaN");
 }

@@ -252,17 +252,17 @@ struct PFinal {   // one output of the finalising launch
 struct PersistDev {
   const InstDesc* desc;  // [n]
   const PSlot* slots;    // [n]
-  const PTask* tasks;    // [n_tasks], the queue order
+  const PTask* tasks;    // the queue order; this launch runs [first, n_tasks)
   int32_t n_tasks, n;
   char* ws;
   int* counters;         // [n] progress, then the next-task counter, then the status word
   long long budget_ns;   // bound of every wait
   int32_t probe_task;    // >= 0: that task waits for a count nothing reaches (timeout check)
-  int32_t pad;
+  int32_t first;
 };
 
-// the persistent launch (grid CTAs; the counters are 0), and the finalising launch over
-// rows[0, n_rows) (gradient rows first: n_grad_rows of them, skipped when grad is null)
+// the persistent launch (grid CTAs; the next-task counter is 0), and the finalising launch
+// over rows[0, n_rows) (gradient rows first: n_grad_rows of them, skipped when grad is null)
 cudaError_t batch_persistent_run(const PersistDev& p, int grid, size_t smem, const double* theta, int64_t ld_theta,
                                  cudaStream_t stream);
 cudaError_t batch_persistent_final(const PersistDev& p, const PFinal* rows, int n_rows, int n_grad_rows,

@@ -866,7 +866,7 @@ cudaError_t sweep_launch(const StreamPlan& sp, const StreamBuffers& b, bool adjo
   p.counters = reinterpret_cast<int*>(static_cast<char*>(b.psi) + sp.counters_off);
   p.budget_ns = 2000000000ll;
   p.probe_task = -1;
-  p.pad = 0;
+  p.first = 0;
   return persistent_sweep_run(p, sp.sweep->grid, theta, stream);
 }
 

@@ -101,3 +101,51 @@ def test_any_wait_that_runs_out_is_reported(routes, which):
     B.energy_grad(theta, e, g, ws)
     B.status(ws)
     _equal_single_calls(insts, e, g)
+
+
+def test_fp64_sweeps_run_together(routes):
+    """Under VQE_FLAG_FP64_SWEEPS every streamed instance that fits a persistent slot is one (H psi
+    on the tensor cores between the two halves of the queue), with the bits of single calls under
+    that flag, for every launch shape, without the gradient, and with a wait that runs out."""
+    insts, B, theta = routes
+    plain, _ = [t.clone() for t in B.energy_grad(theta)]
+    old = vq.set_flags(vq.VQE_FLAG_FP64_SWEEPS)
+    try:
+        gates = sum(insts[i][1].n_params for i in (0, 1, 2, 3, 4))  # all but the resident one
+        assert B.tuning()["n_tasks"] > 2 * gates
+        for shape in ((0, 1024, 128), (1, 256, 128)):
+            B.set_tuning(*shape)
+            e, g = [t.clone() for t in B.energy_grad(theta)]
+            _equal_single_calls(insts, e, g)
+        B.set_tuning(0, 1024, 128)
+        only, _ = B.energy_grad(theta, with_grad=False)
+        assert torch.equal(only, e)
+        ws = vq.alloc_workspace(B.workspace_bytes(True))
+        n = B.tuning()["n_tasks"]
+        for task in (0, n // 3, n - 2, n - 1):  # the last is H psi
+            e2, g2 = torch.zeros_like(e), torch.zeros_like(g)
+            B.set_wait(budget_ns=2_000_000, probe_task=task)
+            try:
+                B.energy_grad(theta, e2, g2, ws)
+                with pytest.raises(vq.VQEError) as ex:
+                    B.status(ws)
+                assert ex.value.code == 4
+            finally:
+                B.set_wait(2_000_000_000, -1)
+            assert torch.isnan(e2[[0, 1, 2, 3, 4]]).all() and torch.equal(e2[5], e[5]), task
+        B.energy_grad(theta, e2, g2, ws)
+        B.status(ws)
+        _equal_single_calls(insts, e2, g2)
+    finally:
+        vq.set_flags(old)
+    again, _ = B.energy_grad(theta)
+    assert torch.equal(again, plain)
+    # a workspace sized without the flag serves a call under it
+    small = vq.alloc_workspace(B.workspace_bytes(True))
+    old = vq.set_flags(vq.VQE_FLAG_FP64_SWEEPS)
+    try:
+        e3, g3 = torch.zeros_like(e), torch.zeros_like(g)
+        B.energy_grad(theta, e3, g3, small)
+        _equal_single_calls(insts, e3, g3)
+    finally:
+        vq.set_flags(old)
