@@ -59,16 +59,17 @@ __global__ void __launch_bounds__(256) k_hop_tables(HopDiag g, int n, int lo_bit
   tab[(size_t(row) << lo_bits) + v] = s;
 }
 
-// lambda = diagonal psi. Consecutive states mostly share the high half.
+// lambda = diagonal psi (0 without a diagonal, also where psi is not finite). Consecutive
+// states mostly share the high half.
 __global__ void __launch_bounds__(256) k_hop_diag(const uint32_t* __restrict__ sector, int64_t D, int lo_bits,
-                                                  const double* __restrict__ tab, const double* __restrict__ psi,
-                                                  double* __restrict__ lam) {
+                                                  int any, const double* __restrict__ tab,
+                                                  const double* __restrict__ psi, double* __restrict__ lam) {
   const uint32_t lo_mask = (1u << lo_bits) - 1u;
   for (int64_t r = blockIdx.x * int64_t(256) + threadIdx.x; r < D; r += int64_t(gridDim.x) * 256) {
     const uint32_t k = __ldg(sector + r), h = k >> lo_bits, v = k & lo_mask;
     double s = tab[v] + tab[(size_t(1) << lo_bits) + h];
     for (uint32_t a = h; a; a &= a - 1) s += tab[(size_t(1 + __ffs(a)) << lo_bits) + v];
-    lam[r] = s * psi[r];
+    lam[r] = any ? s * psi[r] : 0.0;
   }
 }
 
@@ -79,6 +80,7 @@ k_hop_blocks(const HopTables T, const HopStep s, const uint32_t* __restrict__ ra
              const double* __restrict__ psi, double* __restrict__ lam) {
   extern __shared__ __align__(16) double st[];
   double* hop = st + s.most;
+  const uint32_t pad = uint32_t(s.slots) << 16;  // entries from here on are no hops
   const int tid = threadIdx.x;
   const GroupWork w = T.work[s.work0 + blockIdx.x];
   const HopClass c = T.classes[w.cls];
@@ -93,7 +95,6 @@ k_hop_blocks(const HopTables T, const HopStep s, const uint32_t* __restrict__ ra
 #pragma unroll 4
   for (int i = tid; i < total; i += kThreads) copy8(st_a + uint32_t(i) * 8u, psi + rank_of(i, j));
   for (int i = tid; i < s.slots; i += kThreads) hop[i] = vals[__ldg(T.slots + s.slot0 + i)];
-  if (tid == 0) hop[s.slots] = 0.0;  // of the padding entries
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   for (int i = tid; i < total; i += kThreads) {
@@ -107,7 +108,8 @@ k_hop_blocks(const HopTables T, const HopStep s, const uint32_t* __restrict__ ra
 #pragma unroll
       for (int u = 0; u < kAhead; ++u) e[u] = __ldg(list + int64_t(e0 + u) * c.n);
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u) acc = fma(hop[e[u] >> 16], src[e[u] & 0xffffu], acc);
+      for (int u = 0; u < kAhead; ++u)
+        if (e[u] < pad) acc = fma(hop[e[u] >> 16], src[e[u] & 0xffffu], acc);
     }
     lam[r] = before + acc;
   }
@@ -117,7 +119,7 @@ k_hop_blocks(const HopTables T, const HopStep s, const uint32_t* __restrict__ ra
 int hop_width(int w) { return (w + kAhead - 1) / kAhead * kAhead; }
 cudaError_t hop_set_limits() {
   return cudaFuncSetAttribute(k_hop_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (kHopStates + kHopSlots + 1) * 8);
+                              (kHopStates + kHopSlots) * 8);
 }
 
 cudaError_t hop_hpsi(const InstDesc& d, const HopPlan& p, double* tab, const double* psi, double* lam,
@@ -125,9 +127,9 @@ cudaError_t hop_hpsi(const InstDesc& d, const HopPlan& p, double* tab, const dou
   const unsigned size = 1u << d.lo_bits;
   k_hop_tables<<<dim3((size + 255) / 256, unsigned(2 + d.n - d.lo_bits)), 256, 0, stream>>>(p.diag, d.n, d.lo_bits,
                                                                                             d.vals, tab);
-  k_hop_diag<<<stream_grid(d.D), 256, 0, stream>>>(d.sector, d.D, d.lo_bits, tab, psi, lam);
+  k_hop_diag<<<stream_grid(d.D), 256, 0, stream>>>(d.sector, d.D, d.lo_bits, p.diag.slot >= 0 ? 1 : 0, tab, psi, lam);
   for (const HopStep& s : p.steps)
-    k_hop_blocks<<<unsigned(s.ctas), kThreads, size_t(s.most + s.slots + 1) * 8, stream>>>(
+    k_hop_blocks<<<unsigned(s.ctas), kThreads, size_t(s.most + s.slots) * 8, stream>>>(
         p.tables, s, d.rank_hi, d.rank_lo, d.lo_bits, d.vals, psi, lam);
   return cudaGetLastError();
 }

@@ -420,7 +420,7 @@ struct HopTables {
   const GroupWork* work;     // the largest first
   const uint32_t* patterns;  // occupations of the other qubits
   const uint32_t* states;
-  const uint32_t* list;      // value s.slots: 0 (padding)
+  const uint32_t* list;      // value s.slots: padding, no hop
   const int32_t* slots;      // table slot of each value
 };
 struct HopStep {             // one pass
