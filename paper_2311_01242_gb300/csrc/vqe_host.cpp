@@ -1622,7 +1622,7 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
     L.tc.vexp = take(items * 4);
     L.tc.vodd = take(items * 4);
     L.tc.vsum = take(items * 8);
-    L.tc.row = take(Da * 16);
+    L.tc.row = take((Da + 1) * 16);
     L.tc.psi_am = int64_t(L.psi_am);
     L.tc.lam_am = int64_t(L.lam_am);
   }

@@ -130,6 +130,7 @@ struct TcScratch {
   int* vodd;                 // [items]
   double* vsum;              // [items]
   int4* row;                 // [Da] scales of an output row: ea, e, de, flags (bad | odd << 1)
+  int* lost;                 // after them: something is not finite
 };
 struct TcOffsets {           // the same as byte offsets from the workspace's start, and the
   int64_t dig, one_a, one_b, pexp, aexp, ade, bexp, bde, vi, vexp, vodd, vsum, row;
@@ -163,6 +164,10 @@ struct TcCtl {
   bool probe = false;
   long long budget_ns = 0;
 };
+// *lost of an instance, from its workspace offsets
+inline const int* tc_lost(const TcOffsets& off, int Da, const char* ws) {
+  return reinterpret_cast<const int*>(ws + off.row + int64_t(Da) * 16);
+}
 // lam_am (+)= the tensor-core part of H psi_am, for *one or every instance of B
 cudaError_t tc_hpsi(const TcBatch& B, const TcInst* one, char* ws, bool add, const TcCtl& ctl, cudaStream_t stream);
 inline TcBatch tc_single(const TcPlan& tc) {

@@ -654,6 +654,21 @@ k_hpsi_str(const StrPlan sp, const GroupRec* __restrict__ groups, const uint32_t
     hpsi_str_warps<REAL>(sp, int(blockIdx.x) * kStrWarps, groups, emask, vals, psi_am, lam_am, smem);
 }
 
+// The same after the tensor-core H psi, if that met a value that is not finite: its digits make
+// whole rows NaN, where only the outputs that H connects to the value should be.
+template <bool WIDE>
+__global__ void __launch_bounds__(kStrWarps * 32, WIDE ? 4 : 3)
+k_hpsi_str_lost(const int* __restrict__ lost, const StrPlan sp, const GroupRec* __restrict__ groups,
+                const uint32_t* __restrict__ emask, const double* __restrict__ vals,
+                const double* __restrict__ psi_am, double* __restrict__ lam_am) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (*lost == 0) return;
+  if (sp.Db >= kStrMinDb)
+    hpsi_str_row<true, WIDE>(sp, int(blockIdx.x), groups, emask, vals, psi_am, lam_am, smem);
+  else
+    hpsi_str_warps<true>(sp, int(blockIdx.x) * kStrWarps, groups, emask, vals, psi_am, lam_am, smem);
+}
+
 // dst[i] = src[perm[i]] (sector order -> alpha-major) and the reverse scatter
 template <bool REAL>
 __global__ void k_perm_gather(const uint32_t* __restrict__ perm, int64_t D,
@@ -785,6 +800,8 @@ cudaError_t set_str_smem_limit(size_t smem) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hpsi_str<false, false>, a, b);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hpsi_str<true, true>, a, b);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hpsi_str<false, true>, a, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hpsi_str_lost<false>, a, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hpsi_str_lost<true>, a, b);
   return e;
 }
 
@@ -892,9 +909,11 @@ cudaError_t stream_forward(const InstDesc& d, const StreamPlan& sp, const Stream
   return cudaGetLastError();
 }
 
+// any: psi is the caller's and may hold anything (the states of the sweeps are finite, or
+// NaN as a whole)
 template <bool REAL>
 cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuffers& b,
-                        double* energy, cudaStream_t stream) {
+                        double* energy, cudaStream_t stream, bool any = false) {
   typedef typename Amp<REAL>::T T;
   const T* psi = static_cast<const T*>(b.psi);
   T* lam = static_cast<T*>(b.lam);
@@ -924,6 +943,15 @@ cudaError_t stream_hpsi(const InstDesc& d, const StreamPlan& sp, const StreamBuf
         const TcInst one{sp.tc, b.tc, sp.str.ka, sp.str.kb, d.vals};
         const cudaError_t e = tc_hpsi(tc_single(sp.tc), &one, b.base, sp.has_rest, TcCtl{}, stream);
         if (e != cudaSuccess) return e;
+        if (any) {
+          const int* lost = tc_lost(b.tc, sp.tc.Da, b.base);
+          if (sp.str.Db >= kStrWideDb)
+            k_hpsi_str_lost<true><<<str_blocks(sp.str.Da, sp.str.Db), kStrWarps * 32, smem, stream>>>(
+                lost, sp.str, d.groups, d.emask, tv, psi_am, lam_am);
+          else
+            k_hpsi_str_lost<false><<<str_blocks(sp.str.Da, sp.str.Db), kStrWarps * 32, smem, stream>>>(
+                lost, sp.str, d.groups, d.emask, tv, psi_am, lam_am);
+        }
       }
     }
     k_perm_scatter<REAL><<<grid, kStreamThreads, 0, stream>>>(sp.str.perm, d.D, lam_am, lam);
@@ -1012,7 +1040,7 @@ cudaError_t stream_apply_h(const InstDesc& d, const StreamPlan& sp, const Stream
 
 cudaError_t stream_apply_h_real(const InstDesc& d, const StreamPlan& sp, const StreamBuffers& b, double* energy,
                                 cudaStream_t stream) {
-  return stream_hpsi<true>(d, sp, b, energy, stream);
+  return stream_hpsi<true>(d, sp, b, energy, stream, true);
 }
 
 cudaError_t build_hmat(const uint32_t* ellp, int W, int64_t D, const uint32_t* sector, const GroupRec* groups,

@@ -224,6 +224,7 @@ __device__ __forceinline__ TcScratch scratch_of(const TcInst& I, char* ws) {
   s.vodd = reinterpret_cast<int*>(ws + I.off.vodd);
   s.vsum = reinterpret_cast<double*>(ws + I.off.vsum);
   s.row = reinterpret_cast<int4*>(ws + I.off.row);
+  s.lost = reinterpret_cast<int*>(s.row + I.tc.Da);
   return s;
 }
 
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(256) k_tc_values(const TcInst* __restrict__ ma
     sc.vi[int64_t(tc.items + a) * R + m] = bad ? 0 : to_fix(0.5 * (v0 - v1), top);
   }
   if (threadIdx.x == 0) {
+    if (a == 0) *sc.lost = 0;  // the kernels after this one set it
     sc.vexp[a] = bad ? kBadExp : top;
     sc.vodd[a] = odd;
     sc.vsum[a] = sum;
@@ -669,7 +671,10 @@ __global__ void __launch_bounds__(256) k_tc_onespin(const TcInst* __restrict__ m
   __syncthreads();
   if (!beta && w == 7) {
     const int4 scales = row_scales(I.tc, sc, r, lane);
-    if (lane == 0) sc.row[r] = scales;
+    if (lane == 0) {
+      sc.row[r] = scales;
+      if ((scales.w & 1) || sc.pexp[r] == kBadExp) *sc.lost = 1;
+    }
   }
   const int e0 = __ldg(os.off + r), e1 = __ldg(os.off + r + 1);
   int top = -100000;
@@ -726,6 +731,7 @@ __global__ void __launch_bounds__(256) k_tc_onespin(const TcInst* __restrict__ m
   __syncthreads();
   if (tid == 0) {
     for (int i = 1; i < 8; ++i) sum += rs[i];
+    if (bad) *sc.lost = 1;
     oexp[r] = top;
     ode[r] = max(1, exp_above(sum * 1.0001));
   }

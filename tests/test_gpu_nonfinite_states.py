@@ -48,3 +48,27 @@ def test_hops(n, k, diagonal):
         xs, zs, cs = xs[xs != 0], zs[xs != 0], cs[xs != 0]
     H = vq.Hamiltonian(n, xs, zs, cs)
     _same(H, vq.Ansatz(n, (1 << k) - 1, [(0, k)], hcb=True), n + k)
+
+
+def _spin(n_s, na, nb):
+    p = synth.random_problem(np.random.default_rng(100 * n_s + na), n_s, 2, 3)
+    xs, zs, cs = vq.jordan_wigner(n_s, p.h, p.eri)
+    hf = sum(1 << (2 * i) for i in range(na)) | sum(1 << (2 * i + 1) for i in range(nb))
+    return xs, zs, cs, vq.Ansatz(2 * n_s, hf, [[0, 2 * na, -1, -1]])
+
+
+@pytest.mark.parametrize("n_s,na,nb", [(12, 4, 5), (15, 1, 5), (10, 5, 5), (9, 4, 1)])
+def test_tensor_core_strings(n_s, na, nb):
+    """Each form of the string kernel that takes over (many, some and few beta strings)."""
+    xs, zs, cs, A = _spin(n_s, na, nb)
+    _same(vq.Hamiltonian(2 * n_s, xs, zs, cs), A, n_s + na)
+
+
+def test_tensor_core_with_groups_outside_its_form():
+    xs, zs, cs, A = _spin(12, 5, 4)
+    rng = np.random.default_rng(3)
+    ex = [0b101, 0b1010, 0b110011, 0b111100001111]
+    xs = np.concatenate([xs, np.array(ex, dtype=np.uint64)])
+    zs = np.concatenate([zs, rng.integers(0, 1 << 24, size=len(ex)).astype(np.uint64)])
+    cs = np.concatenate([cs, rng.normal(0.0, 0.2, size=len(ex))])
+    _same(vq.Hamiltonian(24, xs, zs, cs), A, 5)
