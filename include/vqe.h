@@ -262,8 +262,14 @@ void vqe_destroy_ansatz(vqe_ansatz_t a);
  * and reduction partials; with VQE_WS_GRAD and real amplitudes, for sectors of
  * 6,000,000 states or more, also the forward sweep's outputs of every
  * (gate, amplitude pair) unit (16 bytes each: 4.5 GB at 30 qubits with 512
- * angles), which the reverse sweep reads (see VQE_FLAG_NO_PHI_STORE). The
- * workspace must be 256-byte aligned.
+ * angles), which the reverse sweep reads (see VQE_FLAG_NO_PHI_STORE). Real
+ * amplitudes of a spin sector with Da alpha and Db beta strings (256 states or
+ * more) also take the operands of H psi on the tensor cores, about 14 bytes for
+ * each entry of a Da x Db, a Da x Da and a Db x Db matrix (the squares at most
+ * 1 GiB, or H psi runs string-driven), and up to 131,072 states, with
+ * VQE_WS_GRAD, 16 bytes for every (gate, amplitude pair) unit. A batch's
+ * workspace holds these for each of its streamed instances that are not
+ * evaluated one by one. The workspace must be 256-byte aligned.
  * The first call for a (Hamiltonian, sector) pair builds that pair's
  * connectivity table (synchronous, allocates); call it before any stream
  * capture. Returns 0 and sets the error message on failure.

@@ -745,7 +745,15 @@ int build_buckets(vqe_hamiltonian_t h, const Strings& S, std::vector<int> keep, 
 // Sectors from this size on run H psi on the tensor cores. Up to kMidStates, where a
 // batch's persistent launch would evaluate them with other kernels than a single
 // call (whose results it equals bit for bit), only without groups outside that form.
+// The digits of the one-spin matrices are dense squares of a spin's strings, far larger
+// than the state where one spin has many strings and the other few (16 orbitals, 8 alpha and
+// 2 beta electrons: 2.3 GB beside 50 MB of vectors): bounded for a single call, and for
+// the instances of a batch, which all have their own, by the state.
 constexpr int64_t kTcMinStates = 256;
+constexpr double kTcOneSpinBytes = double(int64_t(1) << 30), kTcOneSpinPerState = 256.0;
+double tc_one_spin_bytes(size_t Da, size_t Db) {
+  return 2.0 * vqe::kTcDigits * (double(Da) * double((Da + 63) / 64 * 64) + double(Db) * double((Db + 63) / 64 * 64));
+}
 constexpr int64_t kMidStates = int64_t(vqe::kMaxPartials) * vqe::kStreamThreads;
 
 // How the tensor-core H psi takes a group. Amplitudes are multiplied by s(Ia, Ib) =
@@ -871,7 +879,7 @@ int build_one_spin(vqe_hamiltonian_t h, const std::vector<uint32_t>& k, uint32_t
 int build_tc(vqe_hamiltonian_t h, const Strings& S, const std::vector<int>& keep, vqe_hamiltonian_s::Ell* e) {
   const int64_t Da = int64_t(S.ka.size()), Db = int64_t(S.kb.size());
   const int n = h->n;
-  if (Da * Db < kTcMinStates) return VQE_OK;
+  if (Da * Db < kTcMinStates || tc_one_spin_bytes(size_t(Da), size_t(Db)) > kTcOneSpinBytes) return VQE_OK;
   int dev = 0, optin = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
@@ -1563,8 +1571,11 @@ size_t binomial(int n, int k) {
 constexpr int64_t kSweepStates = int64_t(1) << 17;
 bool mid_ansatz(vqe_ansatz_t a) {
   const int64_t D = int64_t(a->sector.size());
-  return a->n_alpha >= 0 && D >= kTcMinStates && D <= kSweepStates && a->M <= 2048 &&
-         int64_t(a->pairs.size()) < (int64_t(1) << 30);
+  if (a->n_alpha < 0 || D < kTcMinStates || D > kSweepStates || a->M > 2048 ||
+      int64_t(a->pairs.size()) >= (int64_t(1) << 30))
+    return false;
+  const size_t Da = binomial(a->n - a->n / 2, a->n_alpha), Db = binomial(a->n / 2, a->n_elec - a->n_alpha);
+  return tc_one_spin_bytes(Da, Db) <= kTcOneSpinPerState * double(D);
 }
 
 // Whether the gate sweeps of this ansatz can run in groups (get_groups). A gate of a spin
@@ -1599,10 +1610,12 @@ WsLayout ws_layout(vqe_ansatz_t a, bool complex_amp, bool with_grad) {
   L.total = L.phi + (keep ? align256(size_t(a->pair_off.empty() ? 0 : a->pair_off.back()) * 16) : 0);
   if (!keep) L.phi = 0;
   std::memset(&L.tc, 0, sizeof(L.tc));
-  L.has_tc = !complex_amp && a->n_alpha >= 0 && int64_t(a->sector.size()) >= kTcMinStates;
+  const int nb = a->n / 2, na = a->n - nb;  // beta and alpha qubits
+  const size_t Da = a->n_alpha < 0 ? 0 : binomial(na, a->n_alpha);
+  const size_t Db = a->n_alpha < 0 ? 0 : binomial(nb, a->n_elec - a->n_alpha);
+  L.has_tc = !complex_amp && a->n_alpha >= 0 && int64_t(a->sector.size()) >= kTcMinStates &&
+             tc_one_spin_bytes(Da, Db) <= kTcOneSpinBytes;
   if (L.has_tc) {
-    const int nb = a->n / 2, na = a->n - nb;  // beta and alpha qubits
-    const size_t Da = binomial(na, a->n_alpha), Db = binomial(nb, a->n_elec - a->n_alpha);
     const size_t DaP = (Da + 63) / 64 * 64, DbP = (Db + 63) / 64 * 64, T = vqe::kTcDigits;
     const size_t items = size_t(na) * size_t(na) + 1, R = size_t((nb * (nb + 1) / 2 + 127) / 128) * 128;
     auto take = [&](size_t bytes) {
