@@ -420,6 +420,8 @@ struct StreamBatch {
   vqe::PSlot* d_slots = nullptr;
   std::unique_ptr<PersistQueue> q[2];     // 0: energy only, 1: with gradient
   size_t counters_off = 0, persist_bytes = 0, big_bytes = 0;
+  size_t energy_bytes = 0;                // of persist_bytes, without the gradient
+  size_t bytes(bool with_grad) const { return with_grad ? persist_bytes : energy_bytes; }
   size_t smem = 0;
   int grid = 0;
   int ctas_per_sm = 0;                    // 0: as many as fit
@@ -3327,7 +3329,15 @@ static int build_mid_batch(vqe_batch_s* B, StreamBatch& sb) {
     const WsLayout L = ws_layout(B->ans[b], false, true);
     sb.mid_off.push_back(off);
     tcs.push_back(tc_inst(B->hams[b], e, L, off));
-    off += L.total;
+    off += L.sw_phi;
+  }
+  // the forward outputs, for gradients only, after everything else
+  sb.energy_bytes = off;
+  std::vector<size_t> phi;
+  for (int i = 0; i < n; ++i) {
+    const WsLayout L = ws_layout(B->ans[sb.mid[size_t(i)]], false, true);
+    phi.push_back(off);
+    off += L.total - L.sw_phi;
   }
   for (int c = 16; c >= 1; c /= 2) {
     vqe::SweepClass k{nullptr, 0, c, 0, !sb.classes.empty(), 0};
@@ -3339,6 +3349,7 @@ static int build_mid_batch(vqe_batch_s* B, StreamBatch& sb) {
       if (!e) return rc;
       sweep.push_back(sweep_inst(B->ans[b], e, B->descs[b], ws_layout(B->ans[b], false, true), sb.mid_off[size_t(i)],
                                  shape[size_t(i)]));
+      sweep.back().phi = int64_t(phi[size_t(i)]);
       sweep.back().task = int32_t(sweep.size()) - 1;
       k.threads = std::max(k.threads, shape[size_t(i)].threads);
       ++k.n;
@@ -3417,7 +3428,7 @@ static int build_stream_batch(vqe_batch_s* B, StreamBatch& sb) {
     sb.pslots.push_back(ps);
   }
   sb.counters_off = off;
-  sb.persist_bytes = off + align256(size_t(n + 3) * sizeof(int));  // and one that stays zero
+  sb.persist_bytes = sb.energy_bytes = off + align256(size_t(n + 3) * sizeof(int));  // and one that stays zero
   int rc;
   if ((rc = build_mid_batch(B, sb))) return rc;
   if (n == 0) return VQE_OK;
@@ -3432,7 +3443,7 @@ static int build_stream_batch(vqe_batch_s* B, StreamBatch& sb) {
     t.off.psi_am = sb.pslots[size_t(s)].psi_am;
     t.off.lam_am = sb.pslots[size_t(s)].lam_am;
     tcs.push_back(t);
-    sb.persist_bytes += L.tc_end - size_t(L.tc.dig);
+    sb.energy_bytes = sb.persist_bytes += L.tc_end - size_t(L.tc.dig);
   }
   if (!tcs.empty() && (rc = build_tc_lists(sb, tcs))) return rc;
   if ((rc = upload(sb.descs, &sb.d_desc))) return rc;
@@ -3527,7 +3538,7 @@ static size_t batch_need(vqe_batch_t b, const StreamBatch& sb, bool with_grad) {
   size_t one = 0;  // largest one-by-one instance
   if (persistent_mode(sb, mode == 0)) {
     for (int i : sb.big) one = std::max(one, ws_layout(b->ans[i], false, with_grad).total);
-    return sb.persist_bytes + one;
+    return sb.bytes(with_grad) + one;
   }
   for (int i : b->streaming[mode]) one = std::max(one, ws_layout(b->ans[i], mode == 1, with_grad).total);
   return one;
@@ -3653,16 +3664,16 @@ static int batch_run(vqe_batch_t b, const double* theta, int64_t ld_theta, doubl
       if ((rc = finish_slots())) return rc;
     } else {
       if ((rc = finish_slots())) return rc;
-      for (size_t k = 0; k < sb.mid.size(); ++k) {
+      for (size_t k = 0; k < sb.mid.size(); ++k) {  // an instance's layout reaches over the next ones'
         const size_t off = sb.mid_off[k];
         rc = run_one_by_one(b, std::vector<int>(1, sb.mid[k]), true, theta, ld_theta, energies, grads, ld_grad,
-                            static_cast<char*>(ws) + off, sb.persist_bytes - off, stream);
+                            static_cast<char*>(ws) + off, sb.bytes(with_grad) - off, stream);
         if (rc) return rc;
       }
     }
     if (!sb.big.empty())
       return run_one_by_one(b, sb.big, true, theta, ld_theta, energies, grads, ld_grad,
-                            static_cast<char*>(ws) + sb.persist_bytes, ws_bytes - sb.persist_bytes, stream);
+                            static_cast<char*>(ws) + sb.bytes(with_grad), ws_bytes - sb.bytes(with_grad), stream);
   } else if (!b->streaming[mode].empty()) {
     if ((rc = check_ws(ws, ws_bytes, batch_need(b, sb, with_grad)))) return rc;
     return run_one_by_one(b, b->streaming[mode], real, theta, ld_theta, energies, grads, ld_grad,
@@ -3858,7 +3869,7 @@ int vqe_batch_status(vqe_batch_t b, const void* ws, size_t ws_bytes, vqe_stream_
   const StreamBatch* last = b->last;
   const StreamBatch& sb = last ? *last : b->sb;
   if (sb.slots.empty() && sb.mid.empty()) return VQE_OK;
-  if (!ws || ws_bytes < sb.persist_bytes) return fail(VQE_ERR_WORKSPACE, "workspace smaller than the batch's");
+  if (!ws || ws_bytes < sb.energy_bytes) return fail(VQE_ERR_WORKSPACE, "workspace smaller than the batch's");
   int status = 0;
   cudaError_t ce = cudaMemcpyAsync(&status, static_cast<const char*>(ws) + sb.counters_off + (sb.slots.size() + 1) * sizeof(int),
                                    sizeof(int), cudaMemcpyDeviceToHost, static_cast<cudaStream_t>(stream));
