@@ -53,7 +53,10 @@ int upload(const std::vector<T>& v, T** out) {
     *out = nullptr;
     return fail(VQE_ERR_NO_MEMORY, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
+  // a copy from pageable memory may return before it has reached the device, and the
+  // streams that read it do not wait for the default one
   e = cudaMemcpy(*out, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
   return VQE_OK;
 }
@@ -3830,6 +3833,7 @@ int vqe_batch_set_tuning(vqe_batch_t b, int ctas_per_sm, int gate_chunk, int swe
       if (!b->res_descs[mode].empty()) {
         cudaError_t e = cudaMemcpy(b->d_res[mode], b->res_descs[mode].data(),
                                    b->res_descs[mode].size() * sizeof(InstDesc), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
       }
     }
