@@ -359,7 +359,11 @@ def run_large(args):
                                "amplitudes)",
                     "q20": f"20 qubits, {p.n_elec} electrons, {len(exc)} UCCSD angles (63,504 sector amplitudes)"
                     }[args.workload]
-        launches = 2 * len(exc) + 8  # trig, init, gates, 4 H psi launches + energy sum, gates, gradient sums
+        # q20: two sweeps, six H psi launches, their dots and the outputs. A launch per gate: trig, init,
+        # gates, eight H psi launches with the permutations, energy sum and its total, gates, gradient sums
+        # (config3, with the kept outputs, one more after H psi that only checks).
+        # q24 sweeps by groups of gates (as many as the draw gives)
+        launches = {"q20": 10, "q24": None, "config3": 2 * len(exc) + 14}.get(args.workload, 2 * len(exc) + 13)
     else:
         insts = [synth.config2_instance(j) for j in range(256)]
         hams = [vq.Hamiltonian.from_problem(p) for p, _, _ in insts]
@@ -536,8 +540,7 @@ def run_adapt(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": pool_profile_traffic(n_pairs), "peak_source": src,
                          "kernel": "k_pool_grad + k_pool_finalize"},
-            "gpu_launches_per_step": 2 * len(exc) + 8, "clocks": clk[0] if clk else None,
-            "clocks_energy_only": clk[1] if len(clk) > 1 else None}
+            "clocks": clk[0] if clk else None, "clocks_energy_only": clk[1] if len(clk) > 1 else None}
     print(json.dumps(line), flush=True)
 
 
@@ -893,14 +896,13 @@ def entry_config3(args, gpu_index):
     assert abs(float(e_np[0]) - e_real) <= 1e-12, "host-buffer and device calls disagree"
     del wsh, B
     peak_hbm, hbm_src = measured_hbm_gbs()
-    # DRAM bytes of one whole evaluation (every kernel, warm L2 as in the timed steps),
-    # else those of the H psi launch alone (cold L2)
-    hpsi_dram = _profile_field("dram_config3_eval.md", RESIDENT_SRC + ["vqe_phi.cu"], "dram_bytes_per_eval")
-    if hpsi_dram is None:
-        hpsi_dram = _profile_field("k_hpsi_str_config3.md", RESIDENT_SRC, "dram_bytes_per_launch")
+    # DRAM bytes of one whole evaluation (every kernel, warm L2 as in the timed steps)
+    hpsi_dram = _profile_field("dram_config3_eval.md", RESIDENT_SRC + ["vqe_phi.cu", "vqe_tc.cu"],
+                               "dram_bytes_per_eval")
     achieved = flops / (ms / 1e3) / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "kernel": "k_hpsi_str (wide block form) + k_gate_fwd/k_gate_adj",
+            "frac": achieved / FP64_PEAK_TFLOPS, "frac_of": "the FP64 peak, for the FP64 operations of the direct sums",
+            "kernel": "k_tc_hops + k_tc_onespin_gemm (tcgen05 fp16 digit products) + k_gate_fwd_keep/k_gate_adj_kept",
             "traffic": hpsi_dram,
             "dram_bytes_per_step": hpsi_dram,
             "hbm_gbs": None if hpsi_dram is None else hpsi_dram / (ms / 1e3) / 1e9,
@@ -908,8 +910,8 @@ def entry_config3(args, gpu_index):
             "hbm_peak": peak_hbm, "hbm_peak_source": hbm_src,
             "state_bytes_per_step": state_bytes, "state_gbs": state_bytes / (ms / 1e3) / 1e9,
             "fp64_flops_per_step": flops, "hpsi_entries": counts["n_entries"], "amplitude_pairs": counts["n_pairs"],
-            "binding": "FP64 pipe and instruction issue of the string-driven H psi (sector-compressed psi and "
-                       "lambda, 72 MB each, stay in L2; DRAM carries the list entries and tables)"}
+            "binding": "H psi: 28 digit products per tile on the tensor cores and their read-out from tensor memory; "
+                       "sweeps: scattered 8-byte accesses of 1,024 gate launches"}
     cpu = cpu_baseline_config3(w, exc)
     return {"workload": "30 qubits, 10 electrons, 512 UCCSD angles (9.0M sector amplitudes), energy + adjoint "
                         "gradient", "metric": "energy+adjoint-grad evals/s", "value": 1e3 / ms, "unit": "evals/s",
@@ -951,10 +953,12 @@ def entry_q20(args, gpu_index):
     ms = tm["ms_per_step"]
     flops, state_bytes = vq.work_estimate(H, A, True)
     peak_hbm, hbm_src = measured_hbm_gbs()
-    dram = _profile_field("dram_q20_eval.md", RESIDENT_SRC, "dram_bytes_per_eval")
+    dram = _profile_field("dram_q20_eval.md", ["vqe_sweep.cu", "vqe_tc.cu", "vqe_device.cuh"], "dram_bytes_per_eval")
     achieved = flops / (ms / 1e3) / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "kernel": "k_hpsi_str (warp form) + k_gate_fwd/k_gate_adj",
+            "frac": achieved / FP64_PEAK_TFLOPS, "frac_of": "the FP64 peak, for the FP64 operations of the direct sums",
+            "kernel": "k_sweep_fwd/k_sweep_rev (one cluster) + k_tc_hops + k_tc_onespin_gemm",
+            "binding": "the chain of gates in cluster shared memory: loads, rotation, stores and a cluster barrier each",
             "traffic": dram, "dram_bytes_per_step": dram,
             "hbm_gbs": None if dram is None else dram / (ms / 1e3) / 1e9,
             "hbm_frac": None if dram is None else dram / (ms / 1e3) / 1e9 / peak_hbm,
@@ -1013,10 +1017,12 @@ def entry_config2(args, gpu_index):
     assert np.abs(e_np - e_dev.cpu().numpy()).max() <= 1e-12, "host-buffer and graph replay disagree"
     del wsh
     peak_hbm, hbm_src = measured_hbm_gbs()
-    dram = _profile_field("k_batch_config2.md", ["vqe_batch.cu", "vqe_device.cuh"], "dram_bytes_per_launch")
+    dram = _profile_field("k_batch_config2.md", ["vqe_sweep.cu", "vqe_tc.cu", "vqe_device.cuh"], "dram_bytes_per_step")
     achieved = flops / (ms / 1e3) / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "kernel": "batched kernels of one graph replay",
+            "frac": achieved / FP64_PEAK_TFLOPS, "frac_of": "the FP64 peak, for the FP64 operations of the direct sums",
+            "kernel": "k_sweep_fwd/k_sweep_rev by cluster size + k_tc_hops + k_tc_onespin_gemm over all instances",
+            "binding": "the longest chain of gates, then H psi of all instances",
             "traffic": dram, "dram_bytes_per_step": dram,
             "hbm_gbs": None if dram is None else dram / (ms / 1e3) / 1e9,
             "hbm_frac": None if dram is None else dram / (ms / 1e3) / 1e9 / peak_hbm,

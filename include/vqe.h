@@ -318,12 +318,18 @@ int vqe_apply_hamiltonian(vqe_hamiltonian_t h, vqe_ansatz_t a, const double* psi
  * sector: psi_dev and lam_dev hold D = sector_dim (vqe_ansatz_info) device
  * doubles, entry r the amplitude of the r-th sector state in increasing order
  * of basis index; energy_dev[0] receives <psi|lambda>. This runs the same
- * real-amplitude H psi kernels as vqe_energy and vqe_energy_grad (string-driven
- * for spin sectors, connectivity rows or a scan of all groups otherwise), which
- * keep the real part of each folded coefficient c * i^{|x&z|}; for the real
- * Hamiltonians of Eq. 2 that is the whole of H. psi_dev and lam_dev must not
- * overlap. workspace: vqe_workspace_bytes(h, a, VQE_WS_ENERGY) bytes,
- * 256-byte aligned. Asynchronous on `stream`.
+ * real-amplitude H psi kernels as vqe_energy and vqe_energy_grad (on the tensor
+ * cores for spin sectors of 256 states or more, string-driven for what they do not
+ * take, by hops for boson sectors above 262,144 states, connectivity rows or a
+ * scan of all groups otherwise), which keep the real part of each folded
+ * coefficient c * i^{|x&z|}; for the real Hamiltonians of Eq. 2 that is the whole
+ * of H. Accuracy: in norm that of FP64 sums. On the tensor cores an entry of
+ * lambda is off by up to 2^-49 of the largest |coefficient| times the largest |psi|
+ * among the terms of its alpha string's row, however small the entry; the other
+ * kernels' error (VQE_FLAG_NO_STRINGS) shrinks with the entry's own terms. An
+ * infinity or NaN in psi reaches the outputs that H connects to it and no others.
+ * psi_dev and lam_dev must not overlap. workspace: vqe_workspace_bytes(h, a,
+ * VQE_WS_ENERGY) bytes, 256-byte aligned. Asynchronous on `stream`.
  */
 int vqe_apply_hamiltonian_sector(vqe_hamiltonian_t h, vqe_ansatz_t a, const double* psi_dev,
                                  double* lam_dev, double* energy_dev, void* workspace,
@@ -530,8 +536,10 @@ int vqe_mlp_adam(int64_t n, float* params, const float* grads, float* m, float* 
  * that every GPU loading this library keeps until the process exits.
  * H psi uses the string or connectivity tables of the (h, sector) pair when an
  * earlier call already built them (vqe_workspace_bytes, vqe_energy_grad or a
- * batch; the results then equal vqe_energy_grad's), else a scan of all X-mask
- * groups per output; the call itself builds nothing.
+ * batch), else a scan of all X-mask groups per output; the call itself builds
+ * nothing. Gates and H psi are FP64 throughout: the results equal
+ * vqe_energy_grad's to rounding (which may sweep in fixed point, and run H psi on
+ * the tensor cores).
  * Limit: instances whose scratch exceeds that size are rejected with
  * VQE_ERR_INVALID_ARG and a message. The scratch is two sector-sized vectors
  * (8-byte real amplitudes, 16-byte complex ones), two more for the string

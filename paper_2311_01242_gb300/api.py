@@ -41,9 +41,8 @@ def _ptr(a):
     return a.ctypes.data
 
 
-# The current stream's handle without the Stream object: torch.cuda.current_stream() takes 8
-# of the 24 us that the smallest call (4 qubits, a 10 us kernel) cost the host
-# (27.5 -> 20.0 us a call).
+# The current stream's handle without the Stream object: torch.cuda.current_stream() took 6 to
+# 8 us of the smallest call (4 qubits, a 10 us kernel: 25.6 -> 19.8 us a call).
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 

@@ -2,14 +2,17 @@
 
 A batch of independent instances (geometries, molecules of uneven size) is
 evaluated by libvqe in one resident launch for the instances that fit shared
-memory and, for the others, in one persistent launch that works through a
+memory; gate sweeps in cluster shared memory around one H psi on the tensor
+cores for mid-size spin sectors; one persistent launch that works through a
 device queue of per-instance tasks (gate rotations on ranges of pairs, H psi on
-ranges of output strings, reductions), plus a small finalising launch.
+ranges of output strings, reductions) for the others of up to 262,144 states;
+the largest one by one.
 GraphBatch captures that launch sequence once and replays it with new angles
 written in place into the captured theta buffer. autotune() times the batch's
 launch shapes (persistent CTAs per SM, amplitude pairs per gate task, resident
-sweep width) and keeps the fastest, cached in a JSON file keyed by the batch's
-sizes; results never depend on the launch shape.
+sweep width; cluster sweeps have no such choice) and keeps the fastest, cached
+in a JSON file keyed by the batch's sizes; results never depend on the launch
+shape.
 """
 import hashlib
 import json

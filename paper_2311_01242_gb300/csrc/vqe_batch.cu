@@ -1,8 +1,12 @@
 // Persistent batched evaluation of many independent instances (the paper runs
 // hundreds of independent simulation jobs over geometries and molecules,
 // abstract and Sec. 4): one launch evaluates E(theta) of Eq. 1 and its adjoint
-// gradient for every streamed instance of a batch, whatever their qubit counts,
-// excitation counts and Hamiltonians.
+// gradient for all instances of a batch that are neither resident nor swept in cluster
+// shared memory (vqe_sweep.cu) and have at most 262,144 states, whatever their qubit
+// counts, excitation counts and Hamiltonians: boson and other electron-number sectors, and
+// spin sectors whose Hamiltonian has groups outside the tensor-core form (vqe_tc.cu). Under
+// VQE_FLAG_FP64_SWEEPS the spin sectors of the tensor-core form too, in two launches
+// around that H psi: tasks [0, split) of the queue, then the rest.
 //
 // The work is a device queue of tasks in a fixed order (built on the host by a
 // list-scheduling pass over cost estimates). Each instance is a chain of

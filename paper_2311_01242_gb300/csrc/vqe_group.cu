@@ -13,13 +13,13 @@
 // per pair; 256 gates took 2.2 ms there. A group of 5 to 6 random double excitations (18
 // pair gates of a boson sector) costs a launch, about 4 us of tables, loads and stores,
 // and per gate shared-memory accesses, 32-bit integer multiply-adds (Q1.62 fixed point:
-// two FP64 operations per clock and SM would take longer) and a block barrier: 0.95 ms
-// at 24 qubits; 2.7 million boson states and 144 gates 4.3 -> 2.2 ms. Issue slots
+// two FP64 operations per clock and SM would take longer) and a block barrier: 0.93 ms
+// at 24 qubits; 2.7 million boson states and 144 gates 4.6 -> 2.6 ms. Issue slots
 // bound the gates of large sectors, latencies the rest. The reverse sweep un-applies psi
 // beside lambda ({psi, lambda} as 16 bytes), so no forward outputs are kept; gradient
-// sums are integers: exact and independent of the order of blocks (cross_add). Tried: 256 threads per
-// CTA (24 qubits 8 % slower), 608 CTAs (10 % slower, nothing of the next launch fits
-// beside them), 5,120 amplitudes per CTA (boson sector 10 % slower), pair lists read
+// sums are integers: exact and independent of the order of blocks (cross_add). Tried: 256
+// threads per CTA (24 qubits 8 % slower), 608 CTAs (10 % slower, nothing of the next launch
+// fits beside them), 5,120 amplitudes per CTA (boson sector 10 % slower), pair lists read
 // from L2 gate by gate (a latency per gate).
 #include <climits>
 #include <cuda_runtime.h>

@@ -748,8 +748,8 @@ int build_buckets(vqe_hamiltonian_t h, const Strings& S, std::vector<int> keep, 
 }
 
 // Sectors from this size on run H psi on the tensor cores. Up to kMidStates, where a
-// batch's persistent launch would evaluate them with other kernels than a single
-// call (whose results it equals bit for bit), only without groups outside that form.
+// batch's persistent launch (under VQE_FLAG_FP64_SWEEPS) runs H psi on them too, only
+// without groups outside that form.
 // The digits of the one-spin matrices are dense squares of a spin's strings, far larger
 // than the state where one spin has many strings and the other few (16 orbitals, 8 alpha and
 // 2 beta electrons: 2.3 GB beside 50 MB of vectors): bounded for a single call, and for
@@ -1181,7 +1181,7 @@ int build_hops(vqe_hamiltonian_t h, vqe_ansatz_t a, vqe_hamiltonian_s::Ell* e) {
     return b;
   };
   // one CTA per SM at least, before fewer passes
-  const size_t bound = std::min(size_t(vqe::kHopStates), std::max<size_t>(D / 152, 1024));
+  const size_t bound = std::min(size_t(vqe::kHopStates), std::max<size_t>(D / (vqe::kGroupCtas / 2), 1024));
   const uint32_t all = uint32_t((uint64_t(1) << n) - 1);
   std::vector<vqe::HopClass> classes;
   std::vector<vqe::GroupWork> work;

@@ -363,7 +363,7 @@ constexpr int kGroupStates = 3456;   // amplitudes per CTA: three or four CTAs p
 constexpr int kGroupPatterns = 256;  // blocks per CTA
 constexpr int kGroupPairs = 8192;    // pair-list entries of a class (all gates of the group)
 constexpr int kGroupGates = 32;      // gates per group
-constexpr int kGroupCtas = 304;      // two per SM: the next group's can start beside them
+constexpr int kGroupCtas = 304;      // two for each of GB300's 152 SMs: the next group's can start beside them
 constexpr int kGroupCopies = 32;     // of the gradient sums, so that blocks rarely meet at one
 struct GroupGate {
   int32_t m;         // angle

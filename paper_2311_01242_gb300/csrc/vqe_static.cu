@@ -21,9 +21,11 @@
 //
 // H psi takes the fastest path that needs no new tables: when an earlier call
 // (vqe_workspace_bytes, vqe_energy_grad, a batch) already built the string or
-// connectivity tables of this (Hamiltonian, sector) pair, they are used, with
-// the same kernels and results as vqe_energy_grad; otherwise every output
-// scans all X-mask groups. The scratch holds only the vectors that path uses.
+// connectivity tables of this (Hamiltonian, sector) pair, they are used;
+// otherwise every output scans all X-mask groups. Gates are one launch each, in
+// FP64. The tensor-core H psi, the hop kernels and the fixed-point sweeps, which
+// vqe_energy_grad takes where they apply, need more scratch, so the results
+// equal its results to rounding. The scratch holds only the vectors that path uses.
 #include <atomic>
 #include <string>
 

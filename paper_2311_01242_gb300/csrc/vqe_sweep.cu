@@ -1,4 +1,4 @@
-// Gate sweeps of mid-size real instances (spin sectors up to 262,144 states), for one
+// Gate sweeps of mid-size real instances (spin sectors of 256 to 131,072 states), for one
 // instance or a batch: the forward sweep and the reverse sweep with the gradient
 // (Sec. 2.1.2's rotations, g_k = 2 <lambda|A_k|phi_k>) as one launch each, a
 // thread-block cluster per instance with the state in the cluster's shared memory.

@@ -25,9 +25,16 @@
 // them per level 2^24 (the levels below 2^-36 may round in their last bit). Levels
 // are combined in 64-bit integers and lambda is accumulated in a per-row fixed point
 // of 62 bits, so no result depends on any order. Measured against the direct sum, H
-// psi alone (one GB300): 85.2 -> 11.1 ms at 30 qubits (9.0M states), 25.0 -> 2.6 ms at
-// 26 qubits and 11 electrons (2.2M), 7.0 -> 0.72 ms at 24 qubits and 10 electrons; the
-// error against 64-bit sums stays that of the direct kernels (2.8e-14 of the norm).
+// psi alone (one GB300): 85.2 -> 15.1 ms at 30 qubits (9.0M states), 25.0 -> 2.9 ms at
+// 26 qubits and 11 electrons (2.2M), 7.0 -> 0.93 ms at 24 qubits and 10 electrons. (The
+// kernels for one instance only, with their plan by value, took 11.1, 2.6 and 0.72 ms: the
+// instance lists of the batch form cost them registers, k_tc_onespin_gemm above all.)
+//
+// In norm the error against 64-bit sums stays that of the direct kernels. Entry by entry
+// it does not follow the entry's size: psi and V are fixed point below their row's largest
+// magnitude, so an entry is off by up to 2^-49 of the largest |V| times the largest |psi|
+// that its row sums (vectors over 26 decades: 2^-48.8 to 2^-49.7), where a direct sum's
+// error shrinks with its terms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -359,8 +366,9 @@ struct TcShared {          // after the operand buffers and the lambda row
 // products. At 30 qubits 7.2 ms: 28 x 4 products of 48 clocks per tile (their shared
 // memory reads bound them at N = 64; 64 clocks would do N = 128), then the read-out,
 // bound by the 16-per-clock float-to-integer conversions. Sixteen reading warps
-// against four: 16.1 -> 7.2 ms, together with products issued from straight-line
-// code.
+// against four: 16.1 -> 7.2 ms, together with products issued from straight-line code. Counters at 24 qubits and 10 electrons (543 us): tensor pipe
+// active 19 % of the cycles, issue slots 34 %, DRAM 15 MB; the rest is waiting between the
+// two, which share the tensor memory.
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_hops(const TcInst* __restrict__ many, const TcInst one, char* ws, const int2* __restrict__ work, int n_work,
           int stages, int lam_len, const TcCtl ctl) {
