@@ -53,12 +53,17 @@ int upload(const std::vector<T>& v, T** out) {
     *out = nullptr;
     return fail(VQE_ERR_NO_MEMORY, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
-  // a copy from pageable memory may return before it has reached the device, and the
-  // streams that read it do not wait for the default one
   e = cudaMemcpy(*out, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
   return VQE_OK;
+}
+
+// After the uploads of an object or of tables: a copy from pageable memory may return
+// before it has reached the device, and the streams that read it do not wait for the
+// default one.
+int settle() {
+  const cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+  return e == cudaSuccess ? VQE_OK : cuda_fail(e, "table upload");
 }
 
 void dfree(void* p) {
@@ -1478,6 +1483,7 @@ const vqe_hamiltonian_s::Ell* get_ell(vqe_hamiltonian_t h, vqe_ansatz_t a, int* 
       e.extra_adds = ex * double(D) / double(sampled);
     }
   }
+  if ((*err = settle()) != VQE_OK) return nullptr;
   auto res = h->ells.emplace(a->key(), e);
   return &res.first->second;
 }
@@ -1747,7 +1753,7 @@ const vqe::SweepPlan* get_sweep(vqe_ansatz_t a) {
   std::vector<InstDesc> dv(1, d);
   std::vector<vqe::PSlot> sv(1, ps);
   ok = ok && upload(dv, &sp->d_desc) == VQE_OK && upload(sv, &sp->d_slot) == VQE_OK &&
-       upload(fwd, &sp->d_fwd) == VQE_OK && (adj.empty() || upload(adj, &sp->d_adj) == VQE_OK);
+       upload(fwd, &sp->d_fwd) == VQE_OK && (adj.empty() || upload(adj, &sp->d_adj) == VQE_OK) && settle() == VQE_OK;
   cudaGetLastError();
   sp->n_fwd = int32_t(fwd.size());
   sp->n_adj = int32_t(adj.size());
@@ -1938,7 +1944,8 @@ const vqe::GroupPlan* get_groups(vqe_ansatz_t a, cudaStream_t stream) {
   };
   const bool ok = pairs.size() < size_t(INT32_MAX) && states.size() < size_t(INT32_MAX) &&
                   vqe::group_set_limits() == cudaSuccess && put(gates, &t.gates) && put(classes, &t.classes) &&
-                  put(work, &t.work) && put(patterns, &t.patterns) && put(ranges, &t.ranges) && put(states, &t.states) && put(pairs, &t.pairs);
+                  put(work, &t.work) && put(patterns, &t.patterns) && put(ranges, &t.ranges) && put(states, &t.states) && put(pairs, &t.pairs) &&
+                  settle() == VQE_OK;
   t.rank_hi = a->d_rank_hi;
   t.rank_lo = a->d_rank_lo;
   t.lo_bits = a->lo_bits;
@@ -2845,6 +2852,7 @@ static int finish_ansatz(std::unique_ptr<vqe_ansatz_s> A, const std::vector<uint
     std::vector<uint2> one2(1, make_uint2(0, 0));
     if ((rc = upload(one2, &A->d_rpairs))) return rc;
   }
+  if ((rc = settle())) return rc;
   A->serial = next_serial();
   *out = A.release();
   return VQE_OK;
@@ -3474,7 +3482,7 @@ static StreamBatch* fp64_batch(vqe_batch_t b, cudaStream_t stream) {
   p->gate_chunk = b->sb.gate_chunk;
   p->budget_ns = b->sb.budget_ns;
   p->probe_task = b->sb.probe_task;
-  if (build_stream_batch(b, *p) != VQE_OK) return nullptr;
+  if (build_stream_batch(b, *p) != VQE_OK || settle() != VQE_OK) return nullptr;
   b->sb64 = std::move(p);
   return b->sb64.get();
 }
@@ -3523,6 +3531,7 @@ int vqe_create_batch(int n_inst, const vqe_hamiltonian_t* hams, const vqe_ansatz
     if (rc) return rc;
   }
   int rc = build_stream_batch(B.get(), B->sb);
+  if (rc == VQE_OK) rc = settle();
   if (rc) return rc;
   *out = B.release();
   return VQE_OK;
@@ -3833,12 +3842,11 @@ int vqe_batch_set_tuning(vqe_batch_t b, int ctas_per_sm, int gate_chunk, int swe
       if (!b->res_descs[mode].empty()) {
         cudaError_t e = cudaMemcpy(b->d_res[mode], b->res_descs[mode].data(),
                                    b->res_descs[mode].size() * sizeof(InstDesc), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
       }
     }
   }
-  return VQE_OK;
+  return settle();
 }
 
 int vqe_batch_get_tuning(vqe_batch_t b, int* ctas_per_sm, int* gate_chunk, int* grid, int64_t* n_tasks) {
