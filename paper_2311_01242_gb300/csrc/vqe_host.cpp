@@ -3487,7 +3487,7 @@ static StreamBatch* fp64_batch(vqe_batch_t b, cudaStream_t stream) {
   return b->sb64.get();
 }
 static bool fp64_differs(vqe_batch_t b) {
-  if ((g_flags & VQE_FLAG_FP64_SWEEPS) == 0) return false;
+  if (!use_real() || (g_flags & VQE_FLAG_FP64_SWEEPS) == 0) return false;
   if (!b->sb.mid.empty()) return true;
   for (int i : b->sb.big)
     if (slot_fits(b->ans[i])) return true;

@@ -14,8 +14,8 @@
 // outputs, phi at that gate, to the workspace (coalesced, 16 bytes per pair), so the
 // reverse sweep keeps lambda only. Gradient contributions are summed as integers:
 // exact, so no result depends on the cluster size or on any order (16 bits of each product
-// below the fixed point's unit are summed beside it: 737 -> 757 us at 16 qubits and 360
-// angles, 760 -> 768 at 20 qubits; without them the gradient lost up to a digit).
+// below the fixed point's unit are summed beside it: 735 -> 742 us at 16 qubits and 360
+// angles, nothing at 20 qubits; without them the gradient lost up to a digit).
 #include <climits>
 #include <cuda_runtime.h>
 
@@ -339,11 +339,8 @@ k_sweep_rev(const SweepInst* __restrict__ many, const SweepInst one, char* ws, c
   int counted = 0;  // pairs of the gate that acc belongs to
   auto add_up = [&](int m) {
     if ((tid & ~31) >= counted) return;
-    const CrossSum s = cross_warp(acc);
-    if (lane == 0) {
-      atomicAdd(gacc + m, static_cast<unsigned long long>(s.hi));
-      atomicAdd(gacc + M + m, static_cast<unsigned long long>(s.lo));
-    }
+    const CrossSum s = cross_warp(acc);  // the same in every lane
+    if (lane < 2) atomicAdd(gacc + (lane ? M + m : m), lane ? s.lo : static_cast<unsigned long long>(s.hi));
   };
   for (int m = M - 1; m >= 0; --m) {
     uint32_t xa[kAhead], xb[kAhead];
